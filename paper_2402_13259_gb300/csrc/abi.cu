@@ -186,7 +186,8 @@ int eulernet::prepare_step_tables(euler_net* h, double dt, double T, cudaStream_
 namespace {
 
 struct Plan {
-  int form = 1, tile_reps = 32, block = 32, grid = 1;
+  int form = 1, tile_reps = 32, block = 32, grid = 1, lanes = 32;
+  bool in_place = false;
   int64_t smem = 0, num_tiles = 0;
   PipePlan pipe;
 };
@@ -213,22 +214,88 @@ bool make_pipe_plan(const euler_net* h, int W, PipePlan* pp) {
   return true;
 }
 
+// Launch shape of the persistent form (tile_slots.cuh) for R replications.
+struct SlotPlan {
+  int Rt = 0, block = 32, lanes = 32;
+  bool in_place = false;  // units with x > m drawn in place
+  int64_t smem = 0, tiles = 0;
+  double fill = 1.0;      // share of the SMs' replication slots in use
+};
+
 bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
 
+
+// One CTA of up to 1024 threads per SM: against two or four smaller ones per
+// SM (each with its own barriers and code position) the 100-station DAG ran
+// 147 and 165 ms instead of 137 (forward, 9,973 replications, 4,000 steps).
+// Tiles are equal, and as many as fill the SMs a whole number of times.
+//
+// Units per warp (lanes): 32 once the SM has 16 warps of them; below, units
+// spread over 16 warps, because a warp runs the union of its lanes' paths
+// (three-station tandem, 1,000 replications: 6.4 ms with one unit to a warp,
+// 8.9 ms with 32).  Units with x > m are drawn in place where the warps take
+// at most 1.5 tasks each in a slot: listing them would add a phase that most
+// warps only wait for (100 stations, 1,200 replications 15.6 -> 12.9 ms; with
+// 1.9 tasks 20.8 ms listed, 24.3 ms in place).
+//
+// Returns false if not even one replication fits a tile.
+bool plan_slots(const euler_net* h, int64_t R, bool grad, int force_Rt, int force_block, SlotPlan* sp) {
+  const int32_t ring = h->tables().ring;
+  auto bytes = [&](int64_t Rt) { return slot_smem_bytes(h->n, h->E, ring, h->n_ex, Rt, grad); };
+  const int64_t limit = h->smem_optin;
+  const int64_t per_rep = (bytes(33) - bytes(1)) / 32;
+  int64_t Rmax = (limit - 256) / per_rep + 1;
+  while (Rmax > 0 && bytes(Rmax) > limit) --Rmax;
+  if (Rmax < 1) return false;
+  const int64_t SM = h->sm_count;
+  auto waves_of = [&](int64_t rt) { return ((R + rt - 1) / rt + SM - 1) / SM; };
+  int64_t Rt = force_Rt;
+  if (Rt <= 0) {
+    // the number of waves w whose smallest even tile costs least: w (Rt + the
+    // replications' worth of a slot's barriers, about 1,000 units)
+    const int64_t w0 = std::max<int64_t>(1, (R + SM * Rmax - 1) / (SM * Rmax));
+    double best = 0.0;
+    for (int64_t w = w0; w <= 2 * w0; ++w) {
+      const int64_t rt = std::max<int64_t>(1, (R + SM * w - 1) / (SM * w));
+      const double cost = (double)waves_of(rt) * ((double)rt + 1000.0 / (double)h->n);
+      if (Rt <= 0 || cost < best) {
+        best = cost;
+        Rt = rt;
+      }
+      if (rt == 1) break;
+    }
+  }
+  if (bytes(Rt) > limit) return false;
+  const int64_t U = (int64_t)h->n * Rt;
+  const int64_t L = std::max<int64_t>(1, std::min<int64_t>(32, (U + 15) / 16));
+  const int64_t tasks = (U + L - 1) / L;
+  sp->Rt = (int)Rt;
+  sp->tiles = (R + Rt - 1) / Rt;
+  sp->smem = bytes(Rt);
+  sp->lanes = (int)L;
+  sp->block = force_block > 0 ? force_block : (int)(32 * std::max<int64_t>(1, std::min<int64_t>(kSlotThreads / 32, tasks)));
+  sp->in_place = 2 * tasks <= 3 * (sp->block / 32);
+  sp->fill = (double)R / (double)(Rt * SM * waves_of(Rt));
+  return true;
+}
+
+// The persistent form runs a slot with one or two block barriers and no launch,
+// state and lists in shared memory; the HBM form's per-step launches spread
+// any replication count evenly over the GPU.  Where a step has work for the
+// whole GPU (n R >= 2^18) the tiles' coarseness decides: with every SM's
+// replication slots in use the persistent form is 1.1 (2,000 stations,
+// s = 10 .. 10,000) to 1.6 times (100 stations) as fast.
+bool hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp) {
+  return (int64_t)h->n * R >= kHbmMinUnitsPerStep && sp.fill < kTileMinFill;
+}
 
 int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
   const int64_t limit = h->smem_optin;
   const int forced_form = (int)h->opt[EULER_OPT_FORM];
-  int Rt = -1;
+  int Rt = 0;  // 0: the planner's choice
   if (h->opt[EULER_OPT_TILE_REPS] > 0) {
     Rt = (int)h->opt[EULER_OPT_TILE_REPS];
     if (!is_pow2(Rt) || Rt > 512) return fail(EULER_ERR_ARG, "tile replications must be a power of two <= 512");
-  } else {
-    for (int cand = 32; cand >= 1; cand >>= 1)
-      if (persistent_smem_bytes(h->n, h->E, h->tables().ring, cand) <= limit) {
-        Rt = cand;
-        break;
-      }
   }
   if (forced_form == 3) {
     const int W = h->opt[EULER_OPT_PIPE_WARPS] > 0 ? (int)h->opt[EULER_OPT_PIPE_WARPS]
@@ -255,15 +322,15 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
     if (forced_form == 3) return fail(EULER_ERR_TOO_LARGE, "pipelined form does not fit");
   }
   pl->form = (forced_form == 1 || forced_form == 2) ? forced_form : 1;
-  // With enough units in one step the HBM form wins: its per-step kernels
-  // balance the stations' uneven sampler work over the whole GPU, where the
-  // persistent form waits at block barriers every phase (forward: every
-  // level), and its state traffic (about 8 + 8 deg bytes per unit) stays far
-  // below HBM bandwidth.  Below the threshold launch gaps dominate.
-  if (forced_form <= 0 && (int64_t)h->n * R >= kHbmMinUnitsPerStep) pl->form = 2;
-  if (pl->form == 1 && (Rt < 1 || persistent_smem_bytes(h->n, h->E, h->tables().ring, Rt) > limit)) {
-    if (forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "network tile does not fit in shared memory");
-    pl->form = 2;
+  SlotPlan sp;
+  if (pl->form == 1) {
+    const int block = h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : 0;
+    const bool tiled = plan_slots(h, R, false, Rt, block, &sp);
+    if (!tiled && forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "network tile does not fit in shared memory");
+    const bool large = forced_form <= 0 && (int64_t)h->n * R >= kHbmMinUnitsPerStep;
+    const bool bad_block = block > 0 && (block % 32 || (Rt > 0 && block % Rt) || block > (large ? 256 : 512));
+    if (!tiled || (forced_form <= 0 && hbm_beats_tiles(h, R, sp)) || (large && bad_block)) pl->form = 2;
+    else if (bad_block) return fail(EULER_ERR_ARG, "block must be a multiple of 32 and of the tile, <= 512");
   }
   if (pl->form == 2) {
     pl->tile_reps = 32;
@@ -274,26 +341,14 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
     pl->num_tiles = (R + 31) / 32;
     return EULER_OK;
   }
-  pl->tile_reps = Rt;
-  const int64_t m_max = scheme == EULER_BACKWARD ? h->n : h->max_level;
-  const int quantum = Rt >= 32 ? 1 : 32 / Rt;  // groups per warp
-  int block;
-  if (h->opt[EULER_OPT_BLOCK] > 0) {
-    block = (int)h->opt[EULER_OPT_BLOCK];
-    if (block % 32 || block % Rt || block > 512) return fail(EULER_ERR_ARG, "block must be a multiple of 32 and of the tile, <= 512");
-  } else {
-    const int64_t gmax = std::max<int64_t>(512 / Rt, 1);
-    const int64_t iters = (m_max + gmax - 1) / gmax;
-    int64_t G = (m_max + iters - 1) / iters;
-    G = (G + quantum - 1) / quantum * quantum;
-    if (G * Rt > 512) G = 512 / Rt;
-    block = (int)std::max<int64_t>(G * Rt, 32);
-  }
-  pl->block = block;
-  pl->smem = persistent_smem_bytes(h->n, h->E, h->tables().ring, Rt);
-  pl->num_tiles = (R + Rt - 1) / Rt;
+  pl->tile_reps = sp.Rt;
+  pl->block = sp.block;
+  pl->lanes = sp.lanes;
+  pl->in_place = sp.in_place;
+  pl->smem = sp.smem;
+  pl->num_tiles = sp.tiles;
   int per_sm = 0;
-  cudaError_t e = persistent_occupancy(scheme, block, (int)pl->smem, &per_sm);
+  cudaError_t e = persistent_occupancy(scheme, pl->block, (int)pl->smem, &per_sm);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
   if (per_sm < 1) {
     if (forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "persistent kernel cannot be resident");
@@ -450,6 +505,50 @@ int eulernet::run_hbm_form(euler_net* h, const NetTables& t, const RunParams& p,
 
 namespace {
 
+// The persistent form's station records (NetTables::rec).  Neighbouring units
+// share a warp, so stations that draw alike stand together: those with
+// external arrivals first, then by flow in classes of a factor of four, by
+// out-degree, and by flow.  (Any order does: in a slot no unit reads what
+// another writes.)
+int upload_records(euler_net* h, const std::vector<int32_t>& level, const std::vector<int32_t>& in_ptr) {
+  const int32_t n = h->n;
+  std::vector<double> flow(n, 0.0);
+  for (int32_t i = 0; i < n; ++i) {
+    if (h->arr_kind == EULER_ARR_SINUSOID) flow[i] = h->w[i] * h->a;
+    if (h->arr_kind == EULER_ARR_TABLE)
+      for (int32_t j = 0; j < h->table_len; ++j) flow[i] += h->table[(int64_t)j * n + i] / h->table_len;
+  }
+  for (int32_t i : h->lvl_station)  // flow order: traffic equations
+    for (int32_t e = h->row_ptr[i]; e < h->row_ptr[i + 1]; ++e) flow[h->col[e]] += flow[i] * h->prob[e];
+  struct Key {
+    int32_t external, flow_class, degree;
+    double flow;
+    int32_t i;
+  };
+  std::vector<Key> order(n);
+  for (int32_t k = 0; k < n; ++k) {
+    const int32_t i = h->lvl_station[k];
+    order[k] = {h->ex_col[i] >= 0 ? 1 : 0, flow[i] > 0.0 ? (int32_t)floor(0.5 * log2(flow[i])) : INT32_MIN,
+                h->row_ptr[i + 1] - h->row_ptr[i], flow[i], i};
+  }
+  std::stable_sort(order.begin(), order.end(), [](const Key& a, const Key& b) {
+    if (a.external != b.external) return a.external > b.external;
+    if (a.flow_class != b.flow_class) return a.flow_class > b.flow_class;
+    if (a.degree != b.degree) return a.degree > b.degree;
+    return a.flow > b.flow;
+  });
+  std::vector<int4> rec(3 * (size_t)n);
+  const int32_t ring = h->tables().ring;
+  for (int32_t k = 0; k < n; ++k) {
+    const int32_t i = order[k].i;
+    rec[3 * (size_t)k] = make_int4(i, level[i], h->ex_col[i], h->servers[i]);
+    rec[3 * (size_t)k + 1] = make_int4(h->row_ptr[i], h->row_ptr[i + 1] - h->row_ptr[i], in_ptr[i], in_ptr[i + 1] - in_ptr[i]);
+    rec[3 * (size_t)k + 2] = make_int4(0, level[i] % ring, 0, 0);
+  }
+  const cudaError_t e = upload(&h->d_rec, rec, &h->h2d_bytes);
+  return e == cudaSuccess ? EULER_OK : cuda_fail(e, "station records");
+}
+
 int validate_net(int32_t n, const int32_t* row_ptr, const int32_t* col, const double* prob,
                  const int32_t* servers, const double* mu, const euler_arrivals* arr,
                  const int32_t* N0) {
@@ -539,6 +638,9 @@ void euler_net_destroy(euler_net* h) {
   cudaFree(h->d_cloc);
   cudaFree(h->d_cpos);
   cudaFree(h->d_csteps);
+  cudaFree(h->d_rec);
+  cudaFree(h->d_tacc);
+  for (unsigned long long* a : h->tacc_old) cudaFree(a);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   delete h;
 }
@@ -674,6 +776,7 @@ int euler_net_create(euler_net** out, int32_t n, const int32_t* row_ptr, const i
     return cuda_fail(e, "euler_net_create upload");
   }
   rc = ensure_levels(h);  // the slot schedules' levels and ring depth
+  if (!rc) rc = upload_records(h, level, in_ptr);
   if (rc) {
     euler_net_destroy(h);
     return rc;
@@ -738,6 +841,54 @@ int euler_net_plan(euler_net* h, int32_t scheme, int64_t R, int32_t* form, int32
 
 namespace {
 
+// The persistent form's per-unit sums for `grid` CTAs, into p.  Grown by
+// doubling and kept until the handle goes: a graph captured from an earlier
+// call may hold the former array, and a call may itself be under capture.
+int slot_scratch(euler_net* h, int grid, int Rt, RunParams* p) {
+  p->acc_stride = slot_acc_len(h->n, h->n_ex, Rt);
+  const size_t need = (size_t)(p->acc_stride * grid);
+  if (need > h->tacc_cap) {
+    const size_t len = std::max(need, 2 * h->tacc_cap);
+    unsigned long long* a = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+    cudaError_t e = cudaMalloc(&a, sizeof(unsigned long long) * len);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return cuda_fail(e, "per-unit sums");
+    if (h->d_tacc) h->tacc_old.push_back(h->d_tacc);
+    h->d_tacc = a;
+    h->tacc_cap = len;
+  }
+  p->acc = h->d_tacc;
+  return EULER_OK;
+}
+
+template <class T>
+int grow(T** p, size_t* cap, size_t need) {
+  if (need <= *cap && *p) return EULER_OK;
+  cudaFree(*p);
+  *p = nullptr;
+  CUDA_TRY(cudaMalloc(p, sizeof(T) * std::max<size_t>(need, 1)));
+  *cap = need;
+  return EULER_OK;
+}
+
+// One launch covers at most about 2e10 station-step updates (about a second),
+// a whole number of waves of tiles.
+template <class Launch>
+cudaError_t launch_tiles(const euler_net* h, RunParams p, int grid, Launch launch) {
+  const int64_t tiles = p.num_tiles;
+  const double wave = (double)h->n * (double)p.tile_reps * (double)p.K * grid;
+  const int64_t step = (int64_t)grid * std::max<int64_t>(1, (int64_t)(2e10 / wave));
+  cudaError_t e = cudaSuccess;
+  for (int64_t t0 = 0; t0 < tiles && e == cudaSuccess; t0 += step) {
+    p.tile0 = t0;
+    p.num_tiles = std::min(tiles, t0 + step);
+    e = launch(p);
+  }
+  return e;
+}
+
 // The run parameters of a plain simulation call (tables current for dt).
 RunParams simulate_params(const euler_net* h, int32_t scheme, double dt, int64_t K, int64_t R, uint64_t seed,
                           int64_t rep_begin, int64_t* stats, int32_t tile_reps, int64_t num_tiles) {
@@ -760,6 +911,11 @@ RunParams simulate_params(const euler_net* h, int32_t scheme, double dt, int64_t
   p.wait_limit = h->opt[EULER_OPT_WAIT_LIMIT] > 0 ? h->opt[EULER_OPT_WAIT_LIMIT] : (int64_t)1 << 25;
   p.test_stall = h->opt[EULER_OPT_TEST_STALL] > 0 ? 1 : 0;
   p.wait_sleep_ns = h->opt[EULER_OPT_WAIT_SLEEP] >= 0 ? (int32_t)std::min<int64_t>(h->opt[EULER_OPT_WAIT_SLEEP], 1000000) : 64;
+  p.task_lanes = 32;
+  p.task_inline = 0;
+  p.tile0 = 0;
+  p.acc = nullptr;
+  p.acc_stride = 0;
   p.muh = h->d_muh;
   p.dep_mode = h->dep_mode();
   p.mtab = h->mtab();
@@ -802,7 +958,7 @@ int euler_net_simulate(euler_net* h, int32_t scheme, double dt, double T, int64_
   Plan pl;
   rc = make_plan(h, scheme, R, &pl);
   if (rc) return rc;
-  const RunParams p = simulate_params(h, scheme, dt, K, R, seed, rep_begin, stats, pl.tile_reps, pl.num_tiles);
+  RunParams p = simulate_params(h, scheme, dt, K, R, seed, rep_begin, stats, pl.tile_reps, pl.num_tiles);
   const NetTables t = h->tables();
   if (pl.form == 3) {
     cudaError_t e = launch_pipeline(t, p, pl.pipe, pl.grid, (int)pl.smem, s);
@@ -810,7 +966,13 @@ int euler_net_simulate(euler_net* h, int32_t scheme, double dt, double T, int64_
     return EULER_OK;
   }
   if (pl.form == 1) {
-    cudaError_t e = launch_persistent(t, p, pl.grid, pl.block, (int)pl.smem, s);
+    p.task_lanes = pl.lanes;
+    p.task_inline = pl.in_place;
+    rc = slot_scratch(h, pl.grid, pl.tile_reps, &p);
+    if (rc) return rc;
+    cudaError_t e = launch_tiles(h, p, pl.grid, [&](const RunParams& pt) {
+      return launch_persistent(t, pt, pl.grid, pl.block, (int)pl.smem, s);
+    });
     if (e != cudaSuccess) return cuda_fail(e, "persistent kernel launch");
     return EULER_OK;
   }
@@ -839,16 +1001,6 @@ void step_mean_grad(const euler_net& h, int32_t i, int64_t tau, double dt, doubl
   g[0] = h.w[i] * ((t1 - t0) + h.b * (c0 - c1) / om);
   g[1] = h.w[i] * h.a * ((c0 - c1) / om);
   g[2] = h.w[i] * h.a * h.b * ((s1 - s0) / om);
-}
-
-template <class T>
-int grow(T** p, size_t* cap, size_t need) {
-  if (need <= *cap && *p) return EULER_OK;
-  cudaFree(*p);
-  *p = nullptr;
-  CUDA_TRY(cudaMalloc(p, sizeof(T) * std::max<size_t>(need, 1)));
-  *cap = need;
-  return EULER_OK;
 }
 
 int refresh_grad_tables(euler_net* h, double dt, double T, cudaStream_t s) {
@@ -912,10 +1064,12 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   const int64_t nb = (R + 31) / 32;
   rc = grow(&h->d_gpartial, &h->gpartial_cap, (size_t)(4 * nb * C + 2 * nb));
   if (rc) return rc;
-  // At scale the HBM form (score sums per station and replication in global
-  // memory, the same step order) is faster, as for euler_net_simulate.
+  // The form as for euler_net_simulate (the HBM form keeps the score sums per
+  // station and replication in global memory, in the same step order).
   const int forced = (int)h->opt[EULER_OPT_FORM];
-  if (forced == 2 || (forced <= 0 && (int64_t)h->n * R >= kHbmMinUnitsPerStep)) {
+  SlotPlan sp;
+  const bool tiled = plan_slots(h, R, true, 0, 0, &sp);
+  if (forced == 2 || (forced <= 0 && (tiled ? hbm_beats_tiles(h, R, sp) : (int64_t)h->n * R >= kHbmMinUnitsPerStep))) {
     const int64_t ld = (R + 3) / 4 * 4;
     rc = grow(&h->d_gmu, &h->gmu_cap, (size_t)(h->n * ld));
     if (rc) return rc;
@@ -961,27 +1115,12 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
     if (e != cudaSuccess) return cuda_fail(e, "gradient reduction launch");
     return EULER_OK;
   }
-  // tile: the largest power of two <= 32 whose state and score sums fit
-  int Rt = 32;
-  int64_t smem = 0;
-  for (; Rt >= 1; Rt /= 2) {
-    smem = persistent_smem_bytes(h->n, h->E, h->tables().ring, Rt) + grad_smem_extra(h->n, h->n_ex, Rt);
-    if (smem <= h->smem_optin) break;
-  }
-  if (Rt < 1) return fail(EULER_ERR_TOO_LARGE, "gradient tile does not fit in shared memory");
-  const int64_t m_max = scheme == EULER_BACKWARD ? h->n : h->max_level;
-  const int quantum = Rt >= 32 ? 1 : 32 / Rt;
-  const int64_t gmax = std::max<int64_t>(512 / Rt, 1);
-  const int64_t iters = (m_max + gmax - 1) / gmax;
-  int64_t G = (m_max + iters - 1) / iters;
-  G = (G + quantum - 1) / quantum * quantum;
-  if (G * Rt > 512) G = 512 / Rt;
-  const int block = (int)std::max<int64_t>(G * Rt, 32);
+  if (!tiled) return fail(EULER_ERR_TOO_LARGE, "gradient tile does not fit in shared memory");
   int per_sm = 0;
-  cudaError_t e = grad_occupancy(scheme, block, (int)smem, &per_sm);
+  cudaError_t e = grad_occupancy(scheme, sp.block, (int)sp.smem, &per_sm);
   if (e != cudaSuccess) return cuda_fail(e, "gradient occupancy query");
   if (per_sm < 1) return fail(EULER_ERR_TOO_LARGE, "gradient kernel cannot be resident");
-  const int64_t tiles = (R + Rt - 1) / Rt;
+  const int64_t tiles = sp.tiles;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * h->sm_count, tiles));
   RunParams p;
   std::memset(&p, 0, sizeof p);
@@ -995,8 +1134,12 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   p.R = R;
   p.rep_begin = rep_begin;
   p.scheme = scheme;
-  p.tile_reps = Rt;
+  p.tile_reps = sp.Rt;
   p.num_tiles = tiles;
+  p.task_lanes = sp.lanes;
+  p.task_inline = sp.in_place;
+  rc = slot_scratch(h, grid, sp.Rt, &p);
+  if (rc) return rc;
   p.cap = h->opt[EULER_OPT_SAMPLER_CAP] > 0 ? (int32_t)h->opt[EULER_OPT_SAMPLER_CAP] : 1000;
   p.stats = stats;
   p.err = h->d_err;
@@ -1008,7 +1151,9 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   p.dep_mode = 0;
   p.mtab = h->mtab();
   CUDA_TRY(cudaMemsetAsync(stats, 0, sizeof(int64_t) * (size_t)euler_stats_len(h->n, R), s));
-  e = launch_persistent_grad(h->tables(), p, grid, block, (int)smem, s);
+  e = launch_tiles(h, p, grid, [&](const RunParams& pt) {
+    return launch_persistent_grad(h->tables(), pt, grid, sp.block, (int)sp.smem, s);
+  });
   if (e != cudaSuccess) return cuda_fail(e, "gradient kernel launch");
   e = launch_grad_reduce(h->n, R, dt, stats, scores, h->d_gpartial, grad, value, grad_var,
                                        h->opt[EULER_OPT_GRAD_CENTER] > 0, s);

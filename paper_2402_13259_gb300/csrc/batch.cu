@@ -12,8 +12,7 @@
 // Rt_j (a power of two) so that its widest phase keeps the block busy
 // (forward: widest level x Rt_j ~ block; backward: all stations), scaled by
 // 2^rt_shift, reduced until its tile's state fits the shared-memory budget;
-// its per-station accumulators go to a global scratch slot of the CTA when
-// they do not fit.  Items are sorted by decreasing cost n_j K_j Rt_j so the
+// its per-unit sums live in the CTA's slot of a global scratch array.  Items are sorted by decreasing cost n_j K_j Rt_j so the
 // last CTAs to finish take the cheapest items.
 //
 // The autotuner searches the persistent launch's threads per block (stations
@@ -64,7 +63,7 @@ struct euler_batch {
   int2* d_items = nullptr;
   size_t items_cap = 0;
   int* d_counter = nullptr;
-  long long* d_sacc = nullptr;
+  unsigned long long* d_sacc = nullptr;  // the CTAs' per-unit sums
   size_t sacc_cap = 0;
   // graph of the last run
   cudaGraphExec_t exec = nullptr;
@@ -97,35 +96,26 @@ int64_t pow2_floor(int64_t v) {
   return p;
 }
 
-int64_t state_bytes(const euler_net* h, int64_t Rt) {
-  return 32 * Rt + 4 * ((int64_t)h->n + (int64_t)h->tables().ring * h->E) * Rt;
+// Shared memory of network j's tile of Rt replications.
+int64_t tile_bytes(const euler_net* h, int64_t Rt) {
+  return slot_smem_bytes(h->n, h->E, h->tables().ring, h->n_ex, Rt, false);
 }
 
 bool runs_hbm(const euler_batch* b, int j) { return b->is_hbm[j] != 0; }
 
 // Tile of network j in the persistent launch: the widest phase x Rt ~ block,
-// scaled by 2^rt_shift, reduced until it fits the budget (per-station sums in
-// shared memory if possible, else in the CTA's global slot).
-bool tile_for(const euler_batch* b, int j, int block, int64_t cap, int rt_shift, int64_t* Rt_out,
-              bool* sacc_global_out) {
+// scaled by 2^rt_shift, reduced until it fits the budget.
+bool tile_for(const euler_batch* b, int j, int block, int64_t cap, int rt_shift, int64_t* Rt_out) {
   const euler_net* h = b->nets[j];
   const int64_t width = b->runs[j].scheme == EULER_BACKWARD ? h->n : h->max_level;
   int64_t Rt = std::max<int64_t>(32, pow2_floor(std::max<int64_t>(block / std::max<int64_t>(width, 1), 1)));
   Rt = rt_shift >= 0 ? Rt << rt_shift : Rt >> -rt_shift;
   Rt = std::max<int64_t>(1, std::min<int64_t>(Rt, block));
-  const int64_t sacc_bytes = 48 * (int64_t)h->n;
-  for (; Rt >= 1; Rt /= 2) {
-    if (256 + sacc_bytes + state_bytes(h, Rt) <= cap) {
+  for (; Rt >= 1; Rt /= 2)
+    if (tile_bytes(h, Rt) <= cap) {
       *Rt_out = Rt;
-      *sacc_global_out = false;
       return true;
     }
-    if (256 + state_bytes(h, Rt) <= cap) {
-      *Rt_out = Rt;
-      *sacc_global_out = true;
-      return true;
-    }
-  }
   return false;
 }
 
@@ -154,13 +144,13 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
   for (int j = 0; j < b->count; ++j)
     b->is_hbm[j] = hbm_min_units > 0 && (int64_t)b->nets[j]->n * b->runs[j].replications >= hbm_min_units;
   std::vector<int64_t> Rt_of(b->count, 1);
-  std::vector<char> sacc_g(b->count, 0);
   for (int j = 0; j < b->count; ++j) {
     if (b->is_hbm[j]) continue;
-    bool g = false;
-    if (!tile_for(b, j, block, cap, rt_shift, &Rt_of[j], &g))
-      return bfail(EULER_ERR_TOO_LARGE, "a network's smallest tile does not fit the shared-memory budget");
-    sacc_g[j] = g;
+    const euler_net* h = b->nets[j];
+    if (288 + 4 * ((int64_t)h->n + (int64_t)h->tables().ring * h->E) > cap)
+      return bfail(EULER_ERR_TOO_LARGE, "a network's state of one replication does not fit the shared-memory budget");
+    // a tile whose lists and arrivals do not fit beside the state: HBM form
+    if (!tile_for(b, j, block, cap, rt_shift, &Rt_of[j])) b->is_hbm[j] = 1;
   }
   if (cp_factor > 0.0) {
     for (int pass = 0; pass < 8; ++pass) {
@@ -169,7 +159,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
       for (int j = 0; j < b->count; ++j) {
         if (b->is_hbm[j]) continue;
         const euler_net* h = b->nets[j];
-        smem = std::max<int64_t>(smem, 256 + (sacc_g[j] ? 0 : 48 * (int64_t)h->n) + state_bytes(h, Rt_of[j]));
+        smem = std::max<int64_t>(smem, tile_bytes(h, Rt_of[j]));
         work += (double)h->n * (double)euler_num_steps(b->runs[j].dt, b->runs[j].T) * (double)b->runs[j].replications;
         n_items += (double)((b->runs[j].replications + Rt_of[j] - 1) / Rt_of[j]);
       }
@@ -205,10 +195,8 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
       continue;
     }
     const int64_t Rt = Rt_of[j];
-    const bool sacc_global = sacc_g[j] != 0;
-    const int64_t sacc_bytes = 48 * (int64_t)h->n;
-    smem = std::max<int64_t>(smem, 256 + (sacc_global ? 0 : sacc_bytes) + state_bytes(h, Rt));
-    if (sacc_global) slot = std::max<int64_t>(slot, 6 * (int64_t)h->n);
+    smem = std::max<int64_t>(smem, tile_bytes(h, Rt));
+    slot = std::max<int64_t>(slot, slot_acc_len(h->n, h->n_ex, Rt));
     RunParams p;
     std::memset(&p, 0, sizeof p);
     p.p0 = h->d_p0;
@@ -228,7 +216,8 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
     p.err = h->d_err;
     p.wait_limit = (int64_t)1 << 25;
     p.test_stall = 0;
-    p.sacc_in_global = sacc_global ? 1 : 0;
+    p.task_lanes = 32;
+    p.task_inline = 0;
     p.muh = h->d_muh;
     p.dep_mode = h->dep_mode();
     p.mtab = h->mtab();
@@ -267,7 +256,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
   if (sacc_need > b->sacc_cap) {
     cudaFree(b->d_sacc);
     b->d_sacc = nullptr;
-    BTRY(cudaMalloc(&b->d_sacc, sizeof(long long) * sacc_need));
+    BTRY(cudaMalloc(&b->d_sacc, sizeof(unsigned long long) * sacc_need));
     b->sacc_cap = sacc_need;
   }
   BTRY(cudaMemcpy(b->d_nets, b->h_nets.data(), sizeof(NetTables) * b->count, cudaMemcpyHostToDevice));

@@ -84,6 +84,11 @@ struct euler_net {
   int64_t* d_racc = nullptr;
   int64_t hbm_cap_ld = 0, hbm_cap_R = 0;
   cudaStream_t cap_stream = nullptr;
+  // persistent form: station records (NetTables::rec) and the CTAs' per-unit sums
+  int4* d_rec = nullptr;
+  unsigned long long* d_tacc = nullptr;
+  size_t tacc_cap = 0;
+  std::vector<unsigned long long*> tacc_old;  // smaller arrays, kept for captured graphs
 
   int64_t opt[13] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
   int64_t h2d_bytes = 0;  // host-to-device bytes copied by this handle so far
@@ -116,15 +121,18 @@ struct euler_net {
     t.ex_col = d_ex_col;
     t.n_ex = n_ex;
     t.pos_level = d_pos_level;
+    t.rec = d_rec;
     t.ring = hbm_depth > 2 ? hbm_depth : 2;
     return t;
   }
 };
 
 namespace eulernet {
-// Units per step (n R) from which the planner takes the HBM form, and its
-// default threads per block.
+// Units per step (n R) from which one step has work for the whole GPU, the
+// share of the SMs' replication slots in use below which the HBM form is then
+// faster than the persistent one, and the HBM form's default threads per block.
 constexpr int64_t kHbmMinUnitsPerStep = int64_t(1) << 18;
+constexpr double kTileMinFill = 0.9;
 constexpr int kHbmBlock = 256;
 // Bytes of HBM-form state per replication chunk, so that a chunk stays in L2.
 constexpr int64_t kHbmL2Budget = int64_t(64) << 20;

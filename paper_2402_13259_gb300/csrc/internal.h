@@ -26,6 +26,9 @@ struct NetTables {
   const int32_t* ex_col;       // [n] column of the station in the Lambda table, or -1
   int32_t n_ex;                // stations with external arrivals
   const int32_t* pos_level;    // [n] level of each position of the level order
+  // [n][3] records of the persistent form's station order: {station, level, ex_col, m_i}, {first edge, edges, first
+  // in-edge, in-edges}, {0, level % ring, 0, 0}
+  const int4* rec;
   int32_t ring;                // routed-count ring slots of the slot schedules:
                                // max(2, largest level gap of an edge + 1)
 };
@@ -40,13 +43,17 @@ struct RunParams {
   int64_t R;          // replications in this call
   int64_t rep_begin;  // global index of local replication 0
   int32_t scheme;     // 0 backward, 1 forward
-  int32_t tile_reps;  // replications per tile (power of two)
+  int32_t tile_reps;  // replications per tile
   int64_t num_tiles;
+  int64_t tile0;      // persistent form: first tile of the launch (num_tiles is one past its last)
   int32_t cap;        // rejection-loop cap
   int64_t wait_limit; // polls of one inter-warp wait before it gives up (pipelined form)
   int32_t wait_sleep_ns; // pause between polls (pipelined form), 0 = none
   int32_t test_stall; // nonzero: no warp publishes progress (tests the timeout path)
-  int32_t sacc_in_global;  // batch kernel: per-station sums in the global scratch slot
+  int32_t task_lanes;      // persistent form: units a warp takes at a time (1 .. 32)
+  int32_t task_inline;     // persistent form: nonzero = units with x > m drawn in place, not listed
+  unsigned long long* acc; // persistent form: per-unit sums, acc_stride entries per CTA
+  int64_t acc_stride;
   const float* muh;      // [n] mu_i dt rounded to float (Eq. (1)/(2) departures)
   int32_t dep_mode;      // 0 exact (Algorithm 1), 1 Eq. (1), 2 Eq. (2)
   const int32_t* mtab;   // [K][n] servers per step (staffing schedule), or nullptr
@@ -69,20 +76,25 @@ inline void set_round_keys(uint32_t* rk, uint32_t key0, uint32_t key1) {
   }
 }
 
-// Shared-memory bytes of the persistent kernel for a tile of `tile_reps`
-// with `ring` slots of routed counts (NetTables::ring for the slot schedules
-// of tile_body, 1 for the step-by-step schedule).
+// Shared-memory bytes of the step-by-step tile kernel (sojourn times) for a
+// tile of `tile_reps` with `ring` slots of routed counts.
 int64_t persistent_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t tile_reps);
+
+// Shared-memory bytes of the persistent kernel (tile_slots.cuh) for a tile of
+// Rt replications, and its per-unit sums (64-bit entries of global scratch per
+// CTA).
+int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad);
+inline int64_t slot_acc_len(int32_t n, int32_t n_ex, int64_t Rt) { return (4 * (int64_t)n + n_ex) * Rt; }
+constexpr int kSlotThreads = 1024;  // most threads per block (the register budget: 64)
 
 // Batched form: one persistent launch over (network, tile) work items.
 cudaError_t batch_occupancy(int block, int smem, int* blocks_per_sm);
 cudaError_t launch_batch(int scheme, bool ext, const NetTables* nets, const RunParams* runs, const int2* items,
-                         int num_items, int* next_item, long long* sacc_scratch,
-                         int64_t sacc_slot_len, int grid, int block, int smem, cudaStream_t s);
+                         int num_items, int* next_item, unsigned long long* acc_scratch,
+                         int64_t acc_slot_len, int grid, int block, int smem, cudaStream_t s);
 
 // Gradient form of the persistent kernel (scores into p.scores) and the
 // fixed-order reduction of L_m(r) S_r over replications.
-int64_t grad_smem_extra(int32_t n, int32_t n_ex, int32_t tile_reps);
 cudaError_t grad_occupancy(int scheme, int block, int smem, int* blocks_per_sm);
 cudaError_t launch_persistent_grad(const NetTables& t, const RunParams& p, int grid, int block,
                                    int smem, cudaStream_t s);

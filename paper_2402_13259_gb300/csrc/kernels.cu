@@ -3,7 +3,8 @@
 // Two forms of the same step (results identical bit for bit):
 //  * persistent: one CTA owns a tile of replications, keeps the whole network
 //    state of the tile (N and the routed edge counts R_e) in shared memory and
-//    runs the time loop inside the kernel; CTAs loop over tiles.
+//    runs the time loop inside the kernel (tile_slots.cuh); CTAs loop over
+//    tiles.
 //  * hbm: state in global memory (station-major, replication-fastest), one
 //    kernel per phase of a step, the step loop captured in a CUDA graph; used
 //    when a tile does not fit in shared memory.
@@ -15,16 +16,12 @@
 //   forward (Sec. 2.2 tasks 1-4, Algorithm 3): level by level in flow order,
 //     gather, external arrivals, D from N_{tau-1} + A^ex + A^in, update,
 //     routing; a barrier between levels.
-// Thread mapping: thread t owns replication slot r = t % Rt of the tile and
-// station slots t / Rt + k G (G = blockDim / Rt), so lanes with consecutive r
-// share a station: per-station sums are warp-segmented reductions and
-// per-replication sums stay in registers.
 #include <cstdint>
 
 #include "internal.h"
 #include "sampling.cuh"
 #include "hbm_step.cuh"
-#include "tile.cuh"
+#include "tile_slots.cuh"
 #include "unit.cuh"
 
 namespace eulernet {
@@ -33,33 +30,19 @@ namespace {
 
 // Single network: CTAs loop over the tiles.
 template <int SCHEME, bool GRAD = false, bool EXT = true>
-__global__ void __launch_bounds__(512, 2) persistent_kernel(NetTables t, const __grid_constant__ RunParams p) {
+__global__ void __launch_bounds__(kSlotThreads, 1)
+    persistent_kernel(const __grid_constant__ NetTables t, const __grid_constant__ RunParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int claim[2];
-  const int32_t n = t.n;
-  const int Rt = p.tile_reps;
-  TileSmem sm;
-  sm.rinv = reinterpret_cast<float*>(smem);
-  sm.sacc = reinterpret_cast<long long*>(smem + 256);
-  sm.racc = sm.sacc + 6 * (int64_t)n;
-  sm.Ns = reinterpret_cast<int32_t*>(sm.racc + 4 * (int64_t)Rt);
-  sm.Rs = sm.Ns + (int64_t)n * Rt;
-  sm.claim = claim;
-  sm.mu_acc = sm.th_acc = nullptr;
-  if (GRAD) {
-    const int64_t end = (int64_t)(reinterpret_cast<unsigned char*>(sm.Rs + (int64_t)t.ring * t.E * Rt) - smem);
-    sm.mu_acc = reinterpret_cast<double*>(smem + (end + 15) / 16 * 16);
-    sm.th_acc = sm.mu_acc + (int64_t)n * Rt;
+  float* rinv = reinterpret_cast<float*>(smem);
+  fill_rinv(rinv);
+  SlotArea sm;
+  sm.rinv = rinv;
+  sm.acc = p.acc + (int64_t)blockIdx.x * p.acc_stride;
+  SamplerCtx cx{rinv, p.cap, 0u};
+  for (int64_t tile = p.tile0 + blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
+    slot_area(t, p.tile_reps, smem + 256, GRAD, sm);
+    tile_slots<SCHEME, GRAD, EXT>(t, p, tile, sm, cx, p.rk);
   }
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  fill_rinv(sm.rinv);
-  for (int64_t k = tid; k < 6 * (int64_t)n; k += nthr) sm.sacc[k] = 0;
-  SamplerCtx cx{sm.rinv, p.cap, 0u};
-  __syncthreads();
-  NoHook hook;
-  for (int64_t tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x)
-    tile_body<SCHEME, GRAD, EXT>(t, p, tile, sm, cx, hook, p.rk);
-  flush_station_sums(t, p, sm.sacc);
   latch(p.err, cx.err);
 }
 
@@ -127,63 +110,41 @@ __global__ void grad_final_kernel(int32_t n, int64_t R, int64_t nb, const double
 
 // Many networks: CTAs take (network, tile) work items from a queue ordered by
 // decreasing cost.  Network j's tables are nets[j], its run runs[j] (tile
-// size, scheme, stats buffer); per-station sums go to shared memory when the
-// network's layout fits (runs[j].sacc_slot < 0) or to the CTA's slot of a
-// global scratch array otherwise.
+// size, scheme, stats buffer), copied to shared memory for the item; the
+// tile's per-unit sums live in the CTA's slot of a global scratch array.
 template <int SCHEME, bool EXT>
-__global__ void __launch_bounds__(512, 2) batch_kernel(const NetTables* nets, const RunParams* runs,
-                                                       const int2* items, int num_items,
-                                                       int* next_item, long long* sacc_scratch,
-                                                       int64_t sacc_slot_len) {
+__global__ void __launch_bounds__(kSlotThreads, 1)
+    batch_kernel(const NetTables* nets, const RunParams* runs, const int2* items, int num_items,
+                 int* next_item, unsigned long long* acc_scratch, int64_t acc_slot_len) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int claim[2];
   __shared__ int s_item;
-  const int tid = threadIdx.x, nthr = blockDim.x;
+  __shared__ __align__(16) unsigned char t_raw[sizeof(NetTables)], p_raw[sizeof(RunParams)];
+  const NetTables& t = *reinterpret_cast<const NetTables*>(t_raw);
+  const RunParams& p = *reinterpret_cast<const RunParams*>(p_raw);
+  const int tid = threadIdx.x;
   float* rinv = reinterpret_cast<float*>(smem);
   fill_rinv(rinv);
+  SlotArea sm;
+  sm.rinv = rinv;
+  sm.acc = acc_scratch + (int64_t)blockIdx.x * acc_slot_len;
   SamplerCtx cx{rinv, 1000, 0u};
-  unsigned err = 0;
-  unsigned* err_ptr = nullptr;
   for (;;) {
     if (tid == 0) s_item = atomicAdd(next_item, 1);
     __syncthreads();
     const int it = s_item;
-    __syncthreads();
     if (it >= num_items) break;
     const int2 wi = items[it];
-    const NetTables t = nets[wi.x];
-    const RunParams p = runs[wi.x];
+    for (int k = tid; k < (int)(sizeof(NetTables) / 4); k += blockDim.x)
+      reinterpret_cast<uint32_t*>(t_raw)[k] = reinterpret_cast<const uint32_t*>(nets + wi.x)[k];
+    for (int k = tid; k < (int)(sizeof(RunParams) / 4); k += blockDim.x)
+      reinterpret_cast<uint32_t*>(p_raw)[k] = reinterpret_cast<const uint32_t*>(runs + wi.x)[k];
+    __syncthreads();
     cx.cap = p.cap;
-    err_ptr = p.err;
-    const int32_t n = t.n;
-    const int Rt = p.tile_reps;
-    TileSmem sm;
-    sm.rinv = rinv;
-    unsigned char* base = smem + 256;
-    if (p.sacc_in_global) {
-      sm.sacc = sacc_scratch + (int64_t)blockIdx.x * sacc_slot_len;
-    } else {
-      sm.sacc = reinterpret_cast<long long*>(base);
-      base += 8 * 6 * (int64_t)n;
-    }
-    sm.racc = reinterpret_cast<long long*>(base);
-    sm.Ns = reinterpret_cast<int32_t*>(sm.racc + 4 * (int64_t)Rt);
-    sm.Rs = sm.Ns + (int64_t)n * Rt;
-    sm.claim = claim;
-    for (int64_t k = tid; k < 6 * (int64_t)n; k += nthr) sm.sacc[k] = 0;
-    __syncthreads();
-    {
-      NoHook hook;
-      tile_body<SCHEME, false, EXT>(t, p, wi.y, sm, cx, hook);
-    }
-    flush_station_sums(t, p, sm.sacc);
-    __syncthreads();
-    err |= cx.err;
+    slot_area(t, p.tile_reps, smem + 256, false, sm);
+    tile_slots<SCHEME, false, EXT>(t, p, wi.y, sm, cx, p.rk);  // ends with a block barrier
+    latch(p.err, cx.err);
     cx.err = 0;
-    if (err && err_ptr) {
-      latch(err_ptr, err);
-      err = 0;
-    }
+    __syncthreads();  // t, p and s_item are rewritten next
   }
 }
 
@@ -248,6 +209,12 @@ int64_t persistent_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t tile_r
          4 * ((int64_t)n + (int64_t)ring * E) * tile_reps;
 }
 
+int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad) {
+  int64_t b = 64 + Rt * (32 + 4 * ((int64_t)n + (int64_t)ring * E + n_ex) + 2 * (int64_t)n);
+  if (grad) b = (b + 15) / 16 * 16 + 8 * Rt * ((int64_t)n + 3 * (int64_t)n_ex);
+  return 256 + b;
+}
+
 namespace {
 bool uses_ext(const RunParams& p) { return p.mtab != nullptr || p.dep_mode != 0; }
 
@@ -303,14 +270,10 @@ cudaError_t batch_occupancy(int block, int smem, int* blocks_per_sm) {
 }
 
 cudaError_t launch_batch(int scheme, bool ext, const NetTables* nets, const RunParams* runs,
-                         const int2* items, int num_items, int* next_item, long long* sacc_scratch,
-                         int64_t sacc_slot_len, int grid, int block, int smem, cudaStream_t s) {
-  void* args[] = {&nets, &runs, &items, &num_items, &next_item, &sacc_scratch, &sacc_slot_len};
+                         const int2* items, int num_items, int* next_item, unsigned long long* acc_scratch,
+                         int64_t acc_slot_len, int grid, int block, int smem, cudaStream_t s) {
+  void* args[] = {&nets, &runs, &items, &num_items, &next_item, &acc_scratch, &acc_slot_len};
   return launch_fn(batch_fn(scheme, ext), args, grid, block, smem, s);
-}
-
-int64_t grad_smem_extra(int32_t n, int32_t n_ex, int32_t tile_reps) {
-  return 16 + 8 * ((int64_t)n + 3 * (int64_t)n_ex) * tile_reps;
 }
 
 cudaError_t grad_occupancy(int scheme, int block, int smem, int* blocks_per_sm) {

@@ -691,19 +691,10 @@ struct BinomialArgs {
   float p;         // the binomial's p in branch 2
 };
 
-// p0c: the constants of p0 = 1 - e^{-mu h} of this station (fixed per call).
-EN_D BinomialArgs departure_branch(int32_t x, int32_t m, float mu, float h, const BinomConst& p0c,
-                                   PhiloxStream& st, SamplerCtx& cx) {
+// The branches with x > m (the caller has tested it).
+EN_D BinomialArgs departure_wait(int32_t x, int32_t m, float mu, float h, PhiloxStream& st,
+                                 SamplerCtx& cx) {
   BinomialArgs b;
-  b.base = 0;
-  b.branch = 0;
-  b.T = 0.0f;
-  b.p = 0.0f;
-  if (EN_LIKELY(x <= m)) {
-    b.n = x;
-    b.c = p0c;
-    return b;
-  }
   const float rate = (float)m * mu;
   PhiloxStream es = st.sibling(2u);
   es.refill();  // every Erlang draw takes at least one word
@@ -713,7 +704,9 @@ EN_D BinomialArgs departure_branch(int32_t x, int32_t m, float mu, float h, cons
   if (T > h) {
     b.n = x - m - 1;
     pb = h / T;
+    b.base = 0;
     b.branch = 1;
+    b.p = 0.0f;
   } else {
     b.n = m;
     b.p = -fm::expm1(-(mu * (h - T)));
@@ -723,6 +716,34 @@ EN_D BinomialArgs departure_branch(int32_t x, int32_t m, float mu, float h, cons
   }
   b.c = binom_const(pb);  // one copy for both branches
   return b;
+}
+
+// p0c: the constants of p0 = 1 - e^{-mu h} of this station (fixed per call).
+EN_D BinomialArgs departure_branch(int32_t x, int32_t m, float mu, float h, const BinomConst& p0c,
+                                   PhiloxStream& st, SamplerCtx& cx) {
+  if (EN_LIKELY(x <= m)) {
+    BinomialArgs b;
+    b.n = x;
+    b.c = p0c;
+    b.base = 0;
+    b.branch = 0;
+    b.T = 0.0f;
+    b.p = 0.0f;
+    return b;
+  }
+  return departure_wait(x, m, mu, h, st, cx);
+}
+
+// d/dmu of the log-probability of the departure draw that took the branch b
+// and its binomial's value v (float32):
+//   x <= m : Bin(x, p0(mu)), dp0/dmu = h(1 - p0)        -> h (k/p0 - x)
+//   x >  m : Erlang(x - m, m mu) density at T            -> (x - m)/mu - m T
+//            plus, if T <= h, Bin(m, p(mu)), dp/dmu = (h - T)(1 - p) -> (h - T)(k/p - m)
+EN_D float departure_score(const BinomialArgs& b, int32_t v, int32_t x, int32_t m, float mu, float h,
+                           float p0) {
+  if (b.branch == 0) return h * ((v > 0 ? (float)v / p0 : 0.0f) - (float)x);
+  const float te = (float)(x - m) / mu - (float)m * b.T;
+  return b.branch == 1 ? te : te + (h - b.T) * ((v > 0 ? (float)v / b.p : 0.0f) - (float)m);
 }
 
 }  // namespace eulernet

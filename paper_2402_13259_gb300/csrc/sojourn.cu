@@ -175,7 +175,6 @@ __global__ void __launch_bounds__(512, 2) sojourn_kernel(NetTables t, RunParams 
   sm.Ns = reinterpret_cast<int32_t*>(sm.racc + 4 * (int64_t)Rt);
   sm.Rs = sm.Ns + (int64_t)n * Rt;
   sm.claim = claim;
-  sm.mu_acc = sm.th_acc = nullptr;
   SojournHook<EXT> hook;
   hook.t = &t;
   hook.p = &p;
@@ -191,7 +190,7 @@ __global__ void __launch_bounds__(512, 2) sojourn_kernel(NetTables t, RunParams 
   SamplerCtx cx{sm.rinv, p.cap, 0u};
   __syncthreads();
   for (int64_t tile = blockIdx.x; tile < p.num_tiles; tile += gridDim.x)
-    tile_body<SCHEME, false, EXT>(t, p, tile, sm, cx, hook);
+    tile_body<SCHEME, EXT>(t, p, tile, sm, cx, hook);
   flush_station_sums(t, p, sm.sacc);
   latch(p.err, cx.err);
 }

@@ -1,0 +1,354 @@
+// tile_slots.cuh -- one tile of replications of the persistent shared-memory
+// form, run slot by slot: the whole time loop of Algorithm 2 (backward) or
+// Algorithm 3 (forward) for Rt replications of one network with the state in
+// shared memory.  Shared by the persistent and the batched kernel.
+//
+// Slots.  Backward, slot tau = 1 .. K+1: every station gathers its routed
+// counts of step tau-1 (ring slot (tau-1) % 2) and completes N_{tau-1}, then
+// draws step tau from it into ring slot tau % 2.  Forward, slot tau = 1 ..
+// K+L-1: the station at level l runs step tau - l, so its predecessors ran
+// that step and it ran its own previous step in earlier slots; routed counts
+// of step s stay in ring slot s % ring until their consumer has read them.
+//
+// What bounds it is instruction issue, and the lanes that wait: a unit with
+// x > m needs an Erlang time and its binomial's constants, several times the
+// work of a unit with x <= m, and on the 100-station DAG 13% of the units are
+// such, spread so that 70% of warps of 32 replications of one station hold at
+// least one.  So each slot has two phases (unless the plan draws all units in
+// place, see plan_slots).  Phase 0 takes the units of the
+// tile 32 to a warp, draws those with x <= m to the end and lists the others
+// in shared memory; phase 1 takes the list 32 to a warp.  One copy of the
+// drawing code serves both.
+//
+// Units are numbered station position x Rt + replication, and a warp takes
+// `task_lanes` consecutive ones, so a tile may have any number of
+// replications (a tile count that divides evenly over the SMs) and a small
+// run can spread its units over more warps, one or a few to each.  Stations
+// are ordered by level and, within one, by the flow through them, so that the
+// units of a warp draw from similar distributions.
+//
+// Statistics: a unit adds its counts to its own 64-bit sums in global memory
+// (reductions without a return value, one address per lane, coalesced); the
+// tile's end sums them over replications and over stations.  Against warp
+// reductions and per-replication sums in each slot this takes no shuffles and
+// leaves the lanes of a warp free to belong to several stations.
+#pragma once
+
+#include <cstdint>
+
+#include "internal.h"
+#include "sampling.cuh"
+#include "unit.cuh"
+
+namespace eulernet {
+
+// A CTA's working area for one tile (see slot_smem_bytes for the layout).
+struct SlotArea {
+  const float* rinv;        // [64] 1/k
+  int* ctr;                 // [8] task and list counters
+  long long* racc;          // [Rt][4] per-replication sums (end of the tile)
+  uint32_t* N;              // [n][Rt] state
+  int32_t* R;               // [ring][E][Rt] routed counts
+  int32_t* aex;             // [n_ex][Rt] arrivals of this slot's listed units (backward)
+  uint16_t* list;           // [n Rt] listed units
+  double* mu_acc;           // GRAD: [n][Rt] score sums in mu_i
+  double* th_acc;           // GRAD: [n_ex][Rt][3] score sums in (a, b, phase)
+  unsigned long long* acc;  // global: [4][n][Rt] sums of N, max(N - m, 0), D, X, then [n_ex][Rt] of A
+};
+
+// Lay the area out from `base` (16-byte aligned) for tiles of Rt replications.
+__device__ __forceinline__ void slot_area(const NetTables& t, int Rt, unsigned char* base, bool grad,
+                                          SlotArea& sm) {
+  const int64_t U = (int64_t)t.n * Rt;
+  sm.ctr = reinterpret_cast<int*>(base);
+  sm.racc = reinterpret_cast<long long*>(base + 64);
+  sm.N = reinterpret_cast<uint32_t*>(sm.racc + 4 * (int64_t)Rt);
+  sm.R = reinterpret_cast<int32_t*>(sm.N + U);
+  sm.aex = sm.R + (int64_t)t.ring * t.E * Rt;
+  sm.list = reinterpret_cast<uint16_t*>(sm.aex + (int64_t)t.n_ex * Rt);
+  sm.mu_acc = sm.th_acc = nullptr;
+  if (grad) {
+    const int64_t end = reinterpret_cast<unsigned char*>(sm.list + U) - base;
+    sm.mu_acc = reinterpret_cast<double*>(base + (end + 15) / 16 * 16);
+    sm.th_acc = sm.mu_acc + U;
+  }
+}
+
+// Sum of a unit's routed-in counts added to s (s <= 2^31 - 1 + 2^30), held at
+// kStateLimit + 1: the caller latches the overflow.
+__device__ __forceinline__ uint32_t slot_gather(const NetTables& t, int32_t k0, int32_t indeg,
+                                                const int32_t* R, int Rt, int r, uint32_t s) {
+  constexpr uint32_t kTop = (uint32_t)kStateLimit + 1u;
+  s = s < kTop ? s : kTop;
+  for (int32_t k = 0; k < indeg; ++k) {
+    s += (uint32_t)R[__ldg(t.in_edge + k0 + k) * Rt + r];
+    s = s < kTop ? s : kTop;
+  }
+  return s;
+}
+
+__device__ __forceinline__ void slot_add(unsigned long long* a, uint32_t v) {
+  if (v) atomicAdd(a, (unsigned long long)v);
+}
+
+// rk: the Philox round keys in the kernel's parameter space (or shared memory).
+template <int SCHEME, bool GRAD, bool EXT>
+__device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& p, int64_t tile,
+                                           const SlotArea& sm, SamplerCtx& cx, const uint32_t* rk) {
+  const int32_t n = t.n;
+  const int64_t r0 = tile * p.tile_reps;
+  const int Rt = (int)(p.R - r0 < p.tile_reps ? p.R - r0 : p.tile_reps);
+  const int U = n * Rt;
+  const int L = p.task_lanes;
+  const uint32_t magic = Rt > 1 ? 0xFFFFFFFFu / (uint32_t)Rt + 1u : 0u;  // q / Rt = umulhi(q, magic), q < 2^16
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
+  const uint32_t rep0 = (uint32_t)(p.rep_begin + r0);
+  unsigned long long* const acc = sm.acc;
+
+  for (int q = tid; q < U; q += nthr) {
+    const int pos = Rt > 1 ? (int)__umulhi((uint32_t)q, magic) : q;
+    sm.N[q] = t.N0 ? (uint32_t)__ldg(t.N0 + __ldg(t.rec + 3 * pos).x) : 0u;
+  }
+  for (int k = tid; k < 4 * Rt; k += nthr) sm.racc[k] = 0;
+  for (int k = tid; k < 4 * U + t.n_ex * Rt; k += nthr) __stcg(acc + k, 0ull);
+  if (GRAD) {
+    for (int q = tid; q < U; q += nthr) sm.mu_acc[q] = 0.0;
+    for (int k = tid; k < 3 * t.n_ex * Rt; k += nthr) sm.th_acc[k] = 0.0;
+  }
+  // ctr[0..1]: tasks handed out in phase 0 (by slot parity), ctr[2]: in phase
+  // 1, ctr[4..6]: listed units (by slot mod 3).  Each is reset in a slot in
+  // which no warp can still read its former value.
+  if (tid < 8) sm.ctr[tid] = tid < 3 ? nwarps : 0;
+  __threadfence();
+  __syncthreads();
+
+  const int last = SCHEME == 0 ? p.K + 1 : p.K + t.L - 1;
+  const int64_t ring_stride = (int64_t)t.E * Rt;
+  int mod_ring = 0, mod3 = 0;
+  const int ntask0 = (U + L - 1) / L;
+  for (int slot = 1; slot <= last; ++slot) {
+    mod_ring = mod_ring + 1 == t.ring ? 0 : mod_ring + 1;
+    mod3 = mod3 == 2 ? 0 : mod3 + 1;
+    int* const count = sm.ctr + 4 + mod3;
+    if (tid == 0) {
+      sm.ctr[(slot + 1) & 1] = nwarps;
+      sm.ctr[2] = nwarps;
+      sm.ctr[4 + (mod3 == 2 ? 0 : mod3 + 1)] = 0;
+    }
+    int ntask = ntask0, listed = U;
+#pragma unroll 1
+    for (int phase = 0; phase < 2; ++phase) {
+      int* const next = phase == 0 ? sm.ctr + (slot & 1) : sm.ctr + 2;
+#pragma unroll 1
+      for (int task = warp; task < ntask;) {
+        const int idx = task * L + lane;
+        bool act = lane < L && idx < listed;
+        bool heavy = false, wait = phase == 1;  // x > m: listed, or drawn here
+        int q = 0, r = 0;
+        int32_t i = 0, tau = 0, ec = -1, m = 0, e0 = 0, deg = 0;
+        uint32_t y = 0, A = 0;
+        int32_t* rcur = sm.R;
+        if (act) {
+          q = phase == 0 ? idx : sm.list[idx];
+          const int pos = Rt > 1 ? (int)__umulhi((uint32_t)q, magic) : q;
+          r = q - pos * Rt;
+          const int4 ra = __ldg(t.rec + 3 * pos), rb = __ldg(t.rec + 3 * pos + 1);
+          i = ra.x;
+          ec = ra.z;
+          m = ra.w;
+          e0 = rb.x;
+          deg = rb.y;
+          if (SCHEME == 0) {
+            tau = slot;
+            rcur = sm.R + (int64_t)(slot & 1) * ring_stride;
+          } else {
+            tau = slot - ra.y;
+            int rs = mod_ring - __ldg(t.rec + 3 * pos + 2).y;
+            rs = rs < 0 ? rs + t.ring : rs;
+            rcur = sm.R + (int64_t)rs * ring_stride;
+            act = tau >= 1 && tau <= p.K;
+          }
+          if (EXT && p.mtab) m = act && tau <= p.K ? __ldg(p.mtab + (int64_t)(tau - 1) * n + i) : m;
+          const uint32_t nprev = sm.N[q];
+          y = nprev;
+          if (act && phase == 0) {
+            const bool draws = SCHEME == 1 || slot <= p.K;
+            if (ec >= 0 && draws) {
+              PhiloxStream arr;
+              arr.init(p.key0, p.key1, 0u, (uint32_t)i, (uint32_t)tau, rep0 + (uint32_t)r, rk);
+              arr.refill();  // every Poisson draw takes at least one word
+              const float lam = __ldg(p.lam + (int64_t)(tau - 1) * t.n_ex + ec);
+              A = (uint32_t)poisson(lam, arr, cx);
+              slot_add(acc + 4 * (int64_t)U + ec * Rt + r, A);
+              if (GRAD && lam > 0.0f) {
+                const float garr = (float)(int32_t)A / lam - 1.0f;
+                if (!isnan(garr)) {
+                  const float* dl = p.dlam + ((int64_t)(tau - 1) * t.n_ex + ec) * 3;
+                  double* th = sm.th_acc + (ec * Rt + r) * 3;
+                  th[0] += (double)(garr * __ldg(dl + 0));
+                  th[1] += (double)(garr * __ldg(dl + 1));
+                  th[2] += (double)(garr * __ldg(dl + 2));
+                }
+              }
+            }
+            if (SCHEME == 1 || slot >= 2) {
+              const int32_t* rin = SCHEME == 1 ? rcur : sm.R + (int64_t)((slot - 1) & 1) * ring_stride;
+              y = slot_gather(t, rb.z, rb.w, rin, Rt, r, SCHEME == 1 ? nprev + A : nprev);
+              if (y > (uint32_t)kStateLimit) {
+                cx.err |= kErrOverflow;
+                y = (uint32_t)kStateLimit;
+              }
+              if (SCHEME == 0) {  // y is N_{tau-1}; its statistics
+                int32_t mp = m;
+                if (EXT && p.mtab) mp = __ldg(p.mtab + (int64_t)(slot - 2) * n + i);
+                atomicAdd(acc + q, (unsigned long long)y);
+                if (y > (uint32_t)mp) slot_add(acc + U + q, y - (uint32_t)mp);
+              }
+            }
+            heavy = draws && (!EXT || p.dep_mode == 0) && y > (uint32_t)m;
+            wait = heavy && p.task_inline != 0;
+            heavy = heavy && p.task_inline == 0;
+            if (!draws) {  // backward, slot K+1: the state is N_K
+              sm.N[q] = y;
+              act = false;
+            }
+            if (heavy) {
+              sm.N[q] = y;
+              if (SCHEME == 0 && ec >= 0) sm.aex[ec * Rt + r] = (int32_t)A;
+              act = false;
+            }
+          }
+        }
+        if (phase == 0) {
+          const unsigned hb = __ballot_sync(kFull, heavy);
+          if (hb) {
+            int at = 0;
+            if (lane == __ffs(hb) - 1) at = atomicAdd(count, __popc(hb));
+            at = __shfl_sync(kFull, at, __ffs(hb) - 1);
+            if (heavy) sm.list[at + __popc(hb & ((1u << lane) - 1u))] = (uint16_t)q;
+          }
+        }
+        if (act) {
+          PhiloxStream svc;
+          svc.init(p.key0, p.key1, 1u, (uint32_t)i, (uint32_t)tau, rep0 + (uint32_t)r, rk);
+          svc.refill();
+          int32_t rem = 0, j0 = -1, D = 0;
+          float smu = 0.0f;
+          BinomialArgs dep;
+          if (SCHEME == 0 && phase == 1 && ec >= 0) A = (uint32_t)sm.aex[ec * Rt + r];
+          if (wait) {
+            dep = departure_wait((int32_t)y, m, __ldg(t.mu + i), p.h, svc, cx);
+          } else {
+            dep.n = (int32_t)y;
+            dep.c = as_const(__ldg(p.p0 + i));
+            dep.base = 0;
+            dep.branch = 0;
+            if (EXT && (p.dep_mode == 1 || (p.dep_mode == 2 && (int32_t)y > m))) {
+              // Eq. (1) (Eq. (2) for x > m): D = min(x, Poisson(min(x, m) mu h))
+              const int32_t b = (int32_t)y < m ? (int32_t)y : m;
+              const int32_t S = poisson((float)b * __ldg(p.muh + i), svc, cx);
+              D = S < (int32_t)y ? S : (int32_t)y;
+              rem = D;
+              j0 = 0;
+            }
+          }
+#pragma unroll 1
+          for (int32_t j = j0; j < deg; ++j) {
+            const int32_t nb = j < 0 ? dep.n : rem;
+            const BinomConst bc = j < 0 ? dep.c : as_const(__ldg(t.qc + e0 + j));
+            const int32_t v = binomial_c(nb, bc, svc, cx);  // Bin(0, .) draws nothing
+            if (j < 0) {
+              D = dep.base + v;
+              rem = D;
+              if (GRAD) smu = departure_score(dep, v, (int32_t)y, m, __ldg(t.mu + i), p.h, __ldg(p.p0f + i));
+            } else {
+              rcur[(e0 + j) * Rt + r] = v;
+              rem = rem - v;
+            }
+          }
+          atomicAdd(acc + 2 * (int64_t)U + q, (unsigned long long)(uint32_t)D);
+          slot_add(acc + 3 * (int64_t)U + q, (uint32_t)rem);
+          if (GRAD) sm.mu_acc[q] += (double)smu;
+          uint32_t nn = y - (uint32_t)D;
+          if (SCHEME == 0) {
+            nn += A;
+            sm.N[q] = nn < 0x7fffffffu ? nn : 0x7fffffffu;
+          } else {
+            sm.N[q] = nn;
+            atomicAdd(acc + q, (unsigned long long)nn);
+            if (nn > (uint32_t)m) slot_add(acc + U + q, nn - (uint32_t)m);
+          }
+        }
+        if (ntask <= nwarps) break;
+        if (lane == 0) task = atomicAdd(next, 1);
+        task = __shfl_sync(kFull, task, 0);
+      }
+      __syncthreads();
+      if (phase == 0) {
+        listed = *count;
+        if (listed == 0) break;  // uniform
+        ntask = (listed + L - 1) / L;
+      }
+    }
+  }
+
+  // The tile's sums: over replications to the stations, over stations to the
+  // replications; N_K from the state.
+  __threadfence();
+  __syncthreads();
+  int64_t* const st_nk = p.stats + 5 * (int64_t)n + 4 * p.R;
+  for (int pos = warp; pos < n; pos += nwarps) {
+    const int4 ra = __ldg(t.rec + 3 * pos);
+    long long s[6] = {0, 0, 0, 0, 0, 0};  // Q, B, D, X, A, N_K
+    for (int r = lane; r < Rt; r += 32) {
+      const int q = pos * Rt + r;
+      const long long Q = (long long)__ldcg(acc + q), W = (long long)__ldcg(acc + U + q);
+      const long long D = (long long)__ldcg(acc + 2 * (int64_t)U + q), X = (long long)__ldcg(acc + 3 * (int64_t)U + q);
+      const long long A = ra.z >= 0 ? (long long)__ldcg(acc + 4 * (int64_t)U + ra.z * Rt + r) : 0;
+      unsigned long long* rr = reinterpret_cast<unsigned long long*>(sm.racc + 4 * r);
+      atomicAdd(rr + 0, (unsigned long long)Q);
+      atomicAdd(rr + 1, (unsigned long long)D);
+      atomicAdd(rr + 2, (unsigned long long)X);
+      if (A) atomicAdd(rr + 3, (unsigned long long)A);
+      s[0] += Q;
+      s[1] += Q - W;
+      s[2] += D;
+      s[3] += X;
+      s[4] += A;
+      s[5] += (long long)sm.N[q];
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const long long v = seg_sum64(s[k], 32);
+      if (lane == 0 && v)
+        atomicAdd(reinterpret_cast<unsigned long long*>(k < 5 ? p.stats + 5 * (int64_t)ra.x + k : st_nk + ra.x),
+                  (unsigned long long)v);
+    }
+  }
+  __syncthreads();
+  int64_t* const st_rep = p.stats + 5 * (int64_t)n + 4 * r0;
+  for (int k = tid; k < 4 * Rt; k += nthr) st_rep[k] = sm.racc[k];
+  if (GRAD) {
+    // S_r: mu_i sums, then (a, b, phase) summed over external stations in order
+    const int64_t C = (int64_t)n + 3;
+    for (int64_t k = tid; k < C * Rt; k += nthr) {
+      const int r = (int)(k % Rt);
+      const int c = (int)(k / Rt);
+      int64_t to;
+      double v;
+      if (c < n) {
+        v = sm.mu_acc[c * Rt + r];
+        to = __ldg(t.rec + 3 * c).x;
+      } else {
+        v = 0.0;
+        for (int32_t ec = 0; ec < t.n_ex; ++ec) v += sm.th_acc[(ec * Rt + r) * 3 + (c - n)];
+        to = c;
+      }
+      p.scores[(r0 + r) * C + to] = v;
+    }
+  }
+  __syncthreads();
+}
+
+}  // namespace eulernet

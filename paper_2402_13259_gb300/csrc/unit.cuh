@@ -129,17 +129,7 @@ __device__ __forceinline__ void serve_and_route(const NetTables& t, const RunPar
       D = dep.base + v;
       rem = D;
       if (GRAD) {
-        // d/dmu_i of the log-probability of this departure (float32):
-        //   x <= m : Bin(x, p0(mu)), dp0/dmu = h(1 - p0)        -> h (k/p0 - x)
-        //   x >  m : Erlang(x - m, m mu) density at T            -> (x - m)/mu - m T
-        //            plus, if T <= h, Bin(m, p(mu)), dp/dmu = (h - T)(1 - p) -> (h - T)(k/p - m)
-        if (dep.branch == 0) {
-          smu = p.h * ((v > 0 ? (float)v / __ldg(p.p0f + i) : 0.0f) - (float)y);
-        } else {
-          const float mu = __ldg(t.mu + i);
-          const float te = (float)(y - m) / mu - (float)m * dep.T;
-          smu = dep.branch == 1 ? te : te + (p.h - dep.T) * ((v > 0 ? (float)v / dep.p : 0.0f) - (float)m);
-        }
+        smu = departure_score(dep, v, y, m, __ldg(t.mu + i), p.h, __ldg(p.p0f + i));
       }
     } else {
       redge[(int64_t)(e0 + j) * stride + col] = v;
