@@ -147,7 +147,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
         bool heavy = false, wait = phase == 1;  // x > m: listed, or drawn here
         int q = 0, r = 0;
         int32_t i = 0, tau = 0, ec = -1, m = 0, e0 = 0, deg = 0;
-        uint32_t y = 0, A = 0;
+        uint32_t y = 0;
         int32_t* rcur = sm.R;
         if (act) {
           q = phase == 0 ? idx : sm.list[idx];
@@ -169,11 +169,12 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
             rcur = sm.R + (int64_t)rs * ring_stride;
             act = tau >= 1 && tau <= p.K;
           }
-          if (EXT && p.mtab) m = act && tau <= p.K ? __ldg(p.mtab + (int64_t)(tau - 1) * n + i) : m;
+          const bool draws = tau <= p.K;
+          if (EXT && p.mtab && act && draws) m = __ldg(p.mtab + (int64_t)(tau - 1) * n + i);
           const uint32_t nprev = sm.N[q];
           y = nprev;
           if (act && phase == 0) {
-            const bool draws = SCHEME == 1 || slot <= p.K;
+            uint32_t A = 0;
             if (ec >= 0 && draws) {
               PhiloxStream arr;
               arr.init(p.key0, p.key1, 0u, (uint32_t)i, (uint32_t)tau, rep0 + (uint32_t)r, rk);
@@ -192,32 +193,29 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
                 }
               }
             }
-            if (SCHEME == 1 || slot >= 2) {
+            if (SCHEME == 1 ? draws : slot >= 2) {
               const int32_t* rin = SCHEME == 1 ? rcur : sm.R + (int64_t)((slot - 1) & 1) * ring_stride;
               y = slot_gather(t, rb.z, rb.w, rin, Rt, r, SCHEME == 1 ? nprev + A : nprev);
               if (y > (uint32_t)kStateLimit) {
                 cx.err |= kErrOverflow;
                 y = (uint32_t)kStateLimit;
               }
-              if (SCHEME == 0) {  // y is N_{tau-1}; its statistics
-                int32_t mp = m;
-                if (EXT && p.mtab) mp = __ldg(p.mtab + (int64_t)(slot - 2) * n + i);
-                atomicAdd(acc + q, (unsigned long long)y);
-                if (y > (uint32_t)mp) slot_add(acc + U + q, y - (uint32_t)mp);
-              }
+            }
+            if (SCHEME == 0 && slot >= 2) {  // y is N_{slot-1}: its statistics
+              const int32_t mp = EXT && p.mtab ? __ldg(p.mtab + (int64_t)(slot - 2) * n + i) : ra.w;
+              atomicAdd(acc + q, (unsigned long long)y);
+              if (y > (uint32_t)mp) slot_add(acc + U + q, y - (uint32_t)mp);
             }
             heavy = draws && (!EXT || p.dep_mode == 0) && y > (uint32_t)m;
             wait = heavy && p.task_inline != 0;
             heavy = heavy && p.task_inline == 0;
-            if (!draws) {  // backward, slot K+1: the state is N_K
-              sm.N[q] = y;
-              act = false;
-            }
-            if (heavy) {
-              sm.N[q] = y;
-              if (SCHEME == 0 && ec >= 0) sm.aex[ec * Rt + r] = (int32_t)A;
-              act = false;
-            }
+            act = draws && !heavy;
+            // backward: the state less this step's departures, a listed unit's
+            // A kept beside it (its x = y is the state without A)
+            if (SCHEME == 0 || heavy) sm.N[q] = y + (SCHEME == 0 ? A : 0u);
+            if (SCHEME == 0 && heavy && ec >= 0) sm.aex[ec * Rt + r] = (int32_t)A;
+          } else if (SCHEME == 0 && act && ec >= 0) {
+            y -= (uint32_t)sm.aex[ec * Rt + r];
           }
         }
         if (phase == 0) {
@@ -233,52 +231,69 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
           PhiloxStream svc;
           svc.init(p.key0, p.key1, 1u, (uint32_t)i, (uint32_t)tau, rep0 + (uint32_t)r, rk);
           svc.refill();
-          int32_t rem = 0, j0 = -1, D = 0;
-          float smu = 0.0f;
-          BinomialArgs dep;
-          if (SCHEME == 0 && phase == 1 && ec >= 0) A = (uint32_t)sm.aex[ec * Rt + r];
+          int32_t D = -1, base = 0, nb = (int32_t)y, branch = 0;
+          float T = 0.0f, pw = 0.0f;
+          BinomConst bc;
           if (wait) {
-            dep = departure_wait((int32_t)y, m, __ldg(t.mu + i), p.h, svc, cx);
+            const BinomialArgs dep = departure_wait((int32_t)y, m, __ldg(t.mu + i), p.h, svc, cx);
+            nb = dep.n;
+            bc = dep.c;
+            base = dep.base;
+            if (GRAD) branch = dep.branch, T = dep.T, pw = dep.p;
           } else {
-            dep.n = (int32_t)y;
-            dep.c = as_const(__ldg(p.p0 + i));
-            dep.base = 0;
-            dep.branch = 0;
+            bc = as_const(__ldg(p.p0 + i));
             if (EXT && (p.dep_mode == 1 || (p.dep_mode == 2 && (int32_t)y > m))) {
               // Eq. (1) (Eq. (2) for x > m): D = min(x, Poisson(min(x, m) mu h))
               const int32_t b = (int32_t)y < m ? (int32_t)y : m;
               const int32_t S = poisson((float)b * __ldg(p.muh + i), svc, cx);
               D = S < (int32_t)y ? S : (int32_t)y;
-              rem = D;
-              j0 = 0;
             }
+          }
+          // One binomial call site draws the departure (base >= 0), then the
+          // row's edges, each pass with constants loaded at the end of the one
+          // before, so the departure's are not live beside them; its sums and
+          // the state are written after the loop (in its first pass they cost
+          // 8%: 100-station DAG backward 351 against 329 ms).
+          int32_t e = e0, re = e0 * Rt + r, rem = 0;
+          const int32_t e1 = e0 + deg;
+          if (EXT && D >= 0) {
+            base = -1;
+            rem = nb = D;
+            if (deg > 0) bc = as_const(__ldg(t.qc + e));
           }
 #pragma unroll 1
-          for (int32_t j = j0; j < deg; ++j) {
-            const int32_t nb = j < 0 ? dep.n : rem;
-            const BinomConst bc = j < 0 ? dep.c : as_const(__ldg(t.qc + e0 + j));
+          while (base >= 0 || e < e1) {
             const int32_t v = binomial_c(nb, bc, svc, cx);  // Bin(0, .) draws nothing
-            if (j < 0) {
-              D = dep.base + v;
-              rem = D;
-              if (GRAD) smu = departure_score(dep, v, (int32_t)y, m, __ldg(t.mu + i), p.h, __ldg(p.p0f + i));
+            if (base >= 0) {
+              rem = base + v;
+              base = -1;
+              if (GRAD) {
+                BinomialArgs dep;
+                dep.branch = branch;
+                dep.T = T;
+                dep.p = pw;
+                sm.mu_acc[q] += (double)departure_score(dep, v, (int32_t)y, m, __ldg(t.mu + i), p.h, __ldg(p.p0f + i));
+              }
+              D = rem;
             } else {
-              rcur[(e0 + j) * Rt + r] = v;
+              rcur[re] = v;
               rem = rem - v;
+              ++e;
+              re += Rt;
             }
+            nb = rem;
+            if (e < e1) bc = as_const(__ldg(t.qc + e));
           }
-          atomicAdd(acc + 2 * (int64_t)U + q, (unsigned long long)(uint32_t)D);
-          slot_add(acc + 3 * (int64_t)U + q, (uint32_t)rem);
-          if (GRAD) sm.mu_acc[q] += (double)smu;
-          uint32_t nn = y - (uint32_t)D;
           if (SCHEME == 0) {
-            nn += A;
-            sm.N[q] = nn < 0x7fffffffu ? nn : 0x7fffffffu;
+            sm.N[q] -= (uint32_t)D;
           } else {
+            const uint32_t nn = y - (uint32_t)D;
             sm.N[q] = nn;
             atomicAdd(acc + q, (unsigned long long)nn);
             if (nn > (uint32_t)m) slot_add(acc + U + q, nn - (uint32_t)m);
           }
+          atomicAdd(acc + 2 * (int64_t)U + q, (unsigned long long)(uint32_t)D);
+          slot_add(acc + 3 * (int64_t)U + q, (uint32_t)rem);
         }
         if (ntask <= nwarps) break;
         if (lane == 0) task = atomicAdd(next, 1);

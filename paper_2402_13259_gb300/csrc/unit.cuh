@@ -107,34 +107,52 @@ __device__ __forceinline__ void serve_and_route(const NetTables& t, const RunPar
   svc.refill();
   const int32_t e0 = __ldg(t.row_ptr + i);
   const int32_t deg = __ldg(t.row_ptr + i + 1) - e0;
-  int32_t rem = 0;
-  int32_t j0 = -1;
+  int32_t rem = 0, base = 0, nb = y, branch = 0;
+  float T = 0.0f, pw = 0.0f;
+  BinomConst bc;
   D = 0;
-  BinomialArgs dep;
   if (EXT && (p.dep_mode == 1 || (p.dep_mode == 2 && y > m))) {
     // Eq. (1) (Eq. (2) for x > m): D = min(x, Poisson(min(x, m) mu h))
     const int32_t b = y < m ? y : m;
     const int32_t S = poisson((float)b * __ldg(p.muh + i), svc, cx);
     D = S < y ? S : y;
-    rem = D;
-    j0 = 0;
+    rem = nb = D;
+    base = -1;
+    if (deg > 0) bc = as_const(__ldg(t.qc + e0));
   } else {
-    dep = departure_branch(y, m, __ldg(t.mu + i), p.h, as_const(__ldg(p.p0 + i)), svc, cx);
+    const BinomialArgs dep = departure_branch(y, m, __ldg(t.mu + i), p.h, as_const(__ldg(p.p0 + i)), svc, cx);
+    nb = dep.n;
+    bc = dep.c;
+    base = dep.base;
+    if (GRAD) branch = dep.branch, T = dep.T, pw = dep.p;
   }
-  for (int32_t j = j0; j < deg; ++j) {
-    const int32_t nb = j < 0 ? dep.n : rem;
-    const BinomConst bc = j < 0 ? dep.c : as_const(__ldg(t.qc + e0 + j));
+  // The departure's pass has base >= 0; each pass loads the next edge's
+  // constants, so nothing of the departure stays live beside them.
+  int32_t e = e0;
+  const int32_t e1 = e0 + deg;
+  int32_t* out = redge + (int64_t)e0 * stride + col;
+#pragma unroll 1
+  while (base >= 0 || e < e1) {
     const int32_t v = binomial_c(nb, bc, svc, cx);  // Bin(0, .) draws nothing
-    if (j < 0) {
-      D = dep.base + v;
+    if (base >= 0) {
+      D = base + v;
       rem = D;
+      base = -1;
       if (GRAD) {
+        BinomialArgs dep;
+        dep.branch = branch;
+        dep.T = T;
+        dep.p = pw;
         smu = departure_score(dep, v, y, m, __ldg(t.mu + i), p.h, __ldg(p.p0f + i));
       }
     } else {
-      redge[(int64_t)(e0 + j) * stride + col] = v;
+      *out = v;
+      out += stride;
       rem = rem - v;
+      ++e;
     }
+    nb = rem;
+    if (e < e1) bc = as_const(__ldg(t.qc + e));
   }
   X = rem;
 }
