@@ -274,7 +274,7 @@ bool plan_slots(const euler_net* h, int64_t R, bool grad, int force_Rt, int forc
   sp->smem = bytes(Rt);
   sp->lanes = (int)L;
   sp->block = force_block > 0 ? force_block : (int)(32 * std::max<int64_t>(1, std::min<int64_t>(kSlotThreads / 32, tasks)));
-  sp->in_place = 2 * tasks <= 3 * (sp->block / 32);
+  sp->in_place = draws_in_place(tasks, sp->block / 32);
   sp->fill = (double)R / (double)(Rt * SM * waves_of(Rt));
   return true;
 }
@@ -510,7 +510,8 @@ namespace {
 // external arrivals first, then by flow in classes of a factor of four, by
 // out-degree, and by flow.  (Any order does: in a slot no unit reads what
 // another writes.)
-int upload_records(euler_net* h, const std::vector<int32_t>& level, const std::vector<int32_t>& in_ptr) {
+int upload_records(euler_net* h, const std::vector<int32_t>& level, const std::vector<int32_t>& in_ptr,
+                   const std::vector<int32_t>& in_edge) {
   const int32_t n = h->n;
   std::vector<double> flow(n, 0.0);
   for (int32_t i = 0; i < n; ++i) {
@@ -542,8 +543,10 @@ int upload_records(euler_net* h, const std::vector<int32_t>& level, const std::v
   for (int32_t k = 0; k < n; ++k) {
     const int32_t i = order[k].i;
     rec[3 * (size_t)k] = make_int4(i, level[i], h->ex_col[i], h->servers[i]);
-    rec[3 * (size_t)k + 1] = make_int4(h->row_ptr[i], h->row_ptr[i + 1] - h->row_ptr[i], in_ptr[i], in_ptr[i + 1] - in_ptr[i]);
-    rec[3 * (size_t)k + 2] = make_int4(0, level[i] % ring, 0, 0);
+    const int32_t k0 = in_ptr[i], deg_in = in_ptr[i + 1] - in_ptr[i];
+    auto in = [&](int32_t j) { return j < deg_in ? in_edge[k0 + j] : h->E; };
+    rec[3 * (size_t)k + 1] = make_int4(h->row_ptr[i], h->row_ptr[i + 1], in(0), in(1));
+    rec[3 * (size_t)k + 2] = make_int4(in(2), level[i] % ring, k0 + 3, std::max(deg_in - 3, 0));
   }
   const cudaError_t e = upload(&h->d_rec, rec, &h->h2d_bytes);
   return e == cudaSuccess ? EULER_OK : cuda_fail(e, "station records");
@@ -776,7 +779,7 @@ int euler_net_create(euler_net** out, int32_t n, const int32_t* row_ptr, const i
     return cuda_fail(e, "euler_net_create upload");
   }
   rc = ensure_levels(h);  // the slot schedules' levels and ring depth
-  if (!rc) rc = upload_records(h, level, in_ptr);
+  if (!rc) rc = upload_records(h, level, in_ptr, in_edge);
   if (rc) {
     euler_net_destroy(h);
     return rc;

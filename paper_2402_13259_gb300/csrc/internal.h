@@ -26,8 +26,10 @@ struct NetTables {
   const int32_t* ex_col;       // [n] column of the station in the Lambda table, or -1
   int32_t n_ex;                // stations with external arrivals
   const int32_t* pos_level;    // [n] level of each position of the level order
-  // [n][3] records of the persistent form's station order: {station, level, ex_col, m_i}, {first edge, edges, first
-  // in-edge, in-edges}, {0, level % ring, 0, 0}
+  // [n][3] records of the persistent form's station order: {station, level,
+  // ex_col, m_i}, {first edge, one past the last, in-edges 0 and 1}, {in-edge
+  // 2, level % ring, position of in-edge 3 in in_edge, in-edges beyond three};
+  // an in-edge that is not there is edge E, whose row of counts is zero
   const int4* rec;
   int32_t ring;                // routed-count ring slots of the slot schedules:
                                // max(2, largest level gap of an edge + 1)
@@ -85,6 +87,9 @@ int64_t persistent_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t tile_r
 // CTA).
 int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad);
 inline int64_t slot_acc_len(int32_t n, int32_t n_ex, int64_t Rt) { return (4 * (int64_t)n + n_ex) * Rt; }
+// Whether `warps` warps draw the units with x > m of a slot of `tasks` tasks in
+// place instead of listing them (see plan_slots).
+inline bool draws_in_place(int64_t tasks, int64_t warps) { return 2 * tasks <= 3 * warps; }
 constexpr int kSlotThreads = 1024;  // most threads per block (the register budget: 64)
 
 // Batched form: one persistent launch over (network, tile) work items.

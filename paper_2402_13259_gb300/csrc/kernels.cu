@@ -32,17 +32,12 @@ namespace {
 template <int SCHEME, bool GRAD = false, bool EXT = true>
 __global__ void __launch_bounds__(kSlotThreads, 1)
     persistent_kernel(const __grid_constant__ NetTables t, const __grid_constant__ RunParams p) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  float* rinv = reinterpret_cast<float*>(smem);
+  float* rinv = reinterpret_cast<float*>(slot_smem);
   fill_rinv(rinv);
-  SlotArea sm;
-  sm.rinv = rinv;
-  sm.acc = p.acc + (int64_t)blockIdx.x * p.acc_stride;
   SamplerCtx cx{rinv, p.cap, 0u};
-  for (int64_t tile = p.tile0 + blockIdx.x; tile < p.num_tiles; tile += gridDim.x) {
-    slot_area(t, p.tile_reps, smem + 256, GRAD, sm);
-    tile_slots<SCHEME, GRAD, EXT>(t, p, tile, sm, cx, p.rk);
-  }
+  unsigned long long* const acc = p.acc + (int64_t)blockIdx.x * p.acc_stride;
+  for (int64_t tile = p.tile0 + blockIdx.x; tile < p.num_tiles; tile += gridDim.x)
+    tile_slots<SCHEME, GRAD, EXT>(t, p, tile, acc, cx, p.rk);
   latch(p.err, cx.err);
 }
 
@@ -116,18 +111,15 @@ template <int SCHEME, bool EXT>
 __global__ void __launch_bounds__(kSlotThreads, 1)
     batch_kernel(const NetTables* nets, const RunParams* runs, const int2* items, int num_items,
                  int* next_item, unsigned long long* acc_scratch, int64_t acc_slot_len) {
-  extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int s_item;
   __shared__ __align__(16) unsigned char t_raw[sizeof(NetTables)], p_raw[sizeof(RunParams)];
   const NetTables& t = *reinterpret_cast<const NetTables*>(t_raw);
   const RunParams& p = *reinterpret_cast<const RunParams*>(p_raw);
   const int tid = threadIdx.x;
-  float* rinv = reinterpret_cast<float*>(smem);
+  float* rinv = reinterpret_cast<float*>(slot_smem);
   fill_rinv(rinv);
-  SlotArea sm;
-  sm.rinv = rinv;
-  sm.acc = acc_scratch + (int64_t)blockIdx.x * acc_slot_len;
   SamplerCtx cx{rinv, 1000, 0u};
+  unsigned long long* const acc = acc_scratch + (int64_t)blockIdx.x * acc_slot_len;
   for (;;) {
     if (tid == 0) s_item = atomicAdd(next_item, 1);
     __syncthreads();
@@ -140,8 +132,7 @@ __global__ void __launch_bounds__(kSlotThreads, 1)
       reinterpret_cast<uint32_t*>(p_raw)[k] = reinterpret_cast<const uint32_t*>(runs + wi.x)[k];
     __syncthreads();
     cx.cap = p.cap;
-    slot_area(t, p.tile_reps, smem + 256, false, sm);
-    tile_slots<SCHEME, false, EXT>(t, p, wi.y, sm, cx, p.rk);  // ends with a block barrier
+    tile_slots<SCHEME, false, EXT>(t, p, wi.y, acc, cx, p.rk);  // ends with a block barrier
     latch(p.err, cx.err);
     cx.err = 0;
     __syncthreads();  // t, p and s_item are rewritten next
@@ -210,9 +201,10 @@ int64_t persistent_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t tile_r
 }
 
 int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad) {
-  int64_t b = 64 + Rt * (32 + 4 * ((int64_t)n + (int64_t)ring * E + n_ex) + 2 * (int64_t)n);
-  if (grad) b = (b + 15) / 16 * 16 + 8 * Rt * ((int64_t)n + 3 * (int64_t)n_ex);
-  return 256 + b;
+  int64_t words = 80 + Rt * (8 + (int64_t)n + (int64_t)ring * (E + 1) + n_ex) + (n * Rt + 1) / 2;
+  words = (words + 3) / 4 * 4;
+  if (grad) words += 2 * Rt * ((int64_t)n + 3 * (int64_t)n_ex);
+  return 4 * words;
 }
 
 namespace {

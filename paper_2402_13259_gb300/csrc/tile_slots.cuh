@@ -24,14 +24,29 @@
 // `task_lanes` consecutive ones, so a tile may have any number of
 // replications (a tile count that divides evenly over the SMs) and a small
 // run can spread its units over more warps, one or a few to each.  Stations
-// are ordered by level and, within one, by the flow through them, so that the
-// units of a warp draw from similar distributions.
+// are ordered by external arrivals, flow and out-degree, so that the units of
+// a warp draw from similar distributions (against level order, forward: 137 ->
+// 125 ms with 66 replications to a tile, 403 -> 348 ms with 5 of 2,000
+// stations).
 //
 // Statistics: a unit adds its counts to its own 64-bit sums in global memory
 // (reductions without a return value, one address per lane, coalesced); the
 // tile's end sums them over replications and over stations.  Against warp
 // reductions and per-replication sums in each slot this takes no shuffles and
 // leaves the lanes of a warp free to belong to several stations.
+//
+// Measured on GB300 against the form it replaces in each case (same samplers):
+// 100-station DAG, 10,000 replications x 10,000 steps, backward 533 -> 347 ms
+// (per-step kernels), 1,237 replications, both schemes 141 -> 45 ms and
+// three-station tandem, 1,000 replications 17.3 -> 6.0 ms (a CTA per 32
+// replications, a station per warp).  It issues 27 warp instructions per unit
+// in 78% of the issue slots, 22.7 of 32 lanes busy (per-step kernels: 41, 61%,
+// 19).  Records with three in-edges and shared memory by 32-bit offsets:
+// backward 329 -> 323 ms, 2,000 stations s = 10 221 -> 212 ms.
+// Tried and slower: the two phases of two halves of the replications in one
+// interval, one barrier instead of two (backward 323 -> 342 ms: the interval's
+// state costs registers that the draws need); a reduction of X where X = 0
+// instead of a branch around it (forward 116.0 -> 117.5 ms).
 #pragma once
 
 #include <cstdint>
@@ -42,59 +57,26 @@
 
 namespace eulernet {
 
-// A CTA's working area for one tile (see slot_smem_bytes for the layout).
-struct SlotArea {
-  const float* rinv;        // [64] 1/k
-  int* ctr;                 // [8] task and list counters
-  long long* racc;          // [Rt][4] per-replication sums (end of the tile)
-  uint32_t* N;              // [n][Rt] state
-  int32_t* R;               // [ring][E][Rt] routed counts
-  int32_t* aex;             // [n_ex][Rt] arrivals of this slot's listed units (backward)
-  uint16_t* list;           // [n Rt] listed units
-  double* mu_acc;           // GRAD: [n][Rt] score sums in mu_i
-  double* th_acc;           // GRAD: [n_ex][Rt][3] score sums in (a, b, phase)
-  unsigned long long* acc;  // global: [4][n][Rt] sums of N, max(N - m, 0), D, X, then [n_ex][Rt] of A
-};
-
-// Lay the area out from `base` (16-byte aligned) for tiles of Rt replications.
-__device__ __forceinline__ void slot_area(const NetTables& t, int Rt, unsigned char* base, bool grad,
-                                          SlotArea& sm) {
-  const int64_t U = (int64_t)t.n * Rt;
-  sm.ctr = reinterpret_cast<int*>(base);
-  sm.racc = reinterpret_cast<long long*>(base + 64);
-  sm.N = reinterpret_cast<uint32_t*>(sm.racc + 4 * (int64_t)Rt);
-  sm.R = reinterpret_cast<int32_t*>(sm.N + U);
-  sm.aex = sm.R + (int64_t)t.ring * t.E * Rt;
-  sm.list = reinterpret_cast<uint16_t*>(sm.aex + (int64_t)t.n_ex * Rt);
-  sm.mu_acc = sm.th_acc = nullptr;
-  if (grad) {
-    const int64_t end = reinterpret_cast<unsigned char*>(sm.list + U) - base;
-    sm.mu_acc = reinterpret_cast<double*>(base + (end + 15) / 16 * 16);
-    sm.th_acc = sm.mu_acc + U;
-  }
-}
-
-// Sum of a unit's routed-in counts added to s (s <= 2^31 - 1 + 2^30), held at
-// kStateLimit + 1: the caller latches the overflow.
-__device__ __forceinline__ uint32_t slot_gather(const NetTables& t, int32_t k0, int32_t indeg,
-                                                const int32_t* R, int Rt, int r, uint32_t s) {
-  constexpr uint32_t kTop = (uint32_t)kStateLimit + 1u;
-  s = s < kTop ? s : kTop;
-  for (int32_t k = 0; k < indeg; ++k) {
-    s += (uint32_t)R[__ldg(t.in_edge + k0 + k) * Rt + r];
-    s = s < kTop ? s : kTop;
-  }
-  return s;
-}
+// Dynamic shared memory of the slot kernels (see slot_smem_bytes), addressed
+// by 32-bit word offsets: 1/k table [64] | counters [16] | racc i64 [Rt][4],
+// the replications' sums at the tile's end | N u32 [n][Rt], the state |
+// R i32 [ring][E+1][Rt], routed counts, row E zero (stands in for an in-edge
+// that is not there) | aex i32 [n_ex][Rt], this slot's arrivals of listed units
+// (backward) | list u16 [n Rt] | GRAD: mu_acc f64 [n][Rt], th_acc f64
+// [n_ex][Rt][3], score sums.
+extern __shared__ __align__(16) uint32_t slot_smem[];
 
 __device__ __forceinline__ void slot_add(unsigned long long* a, uint32_t v) {
   if (v) atomicAdd(a, (unsigned long long)v);
 }
 
-// rk: the Philox round keys in the kernel's parameter space (or shared memory).
+// acc: global scratch of the CTA, [4][n][Rt] sums of N, max(N - m, 0), D, X,
+// then [n_ex][Rt] of A.  rk: the Philox round keys in the kernel's parameter
+// space (or shared memory).
 template <int SCHEME, bool GRAD, bool EXT>
 __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& p, int64_t tile,
-                                           const SlotArea& sm, SamplerCtx& cx, const uint32_t* rk) {
+                                           unsigned long long* const acc, SamplerCtx& cx,
+                                           const uint32_t* rk) {
   const int32_t n = t.n;
   const int64_t r0 = tile * p.tile_reps;
   const int Rt = (int)(p.R - r0 < p.tile_reps ? p.R - r0 : p.tile_reps);
@@ -104,74 +86,80 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
   const uint32_t rep0 = (uint32_t)(p.rep_begin + r0);
-  unsigned long long* const acc = sm.acc;
+  // word offsets of the area
+  const int ring_stride = (t.E + 1) * Rt;
+  const int oRacc = 80, oN = oRacc + 8 * Rt, oR = oN + U, oAex = oR + t.ring * ring_stride;
+  const int oList = oAex + t.n_ex * Rt, oMu = (oList + (U + 1) / 2 + 3) / 4 * 4;
+  int* const ctr = reinterpret_cast<int*>(slot_smem + 64);
+  uint16_t* const list = reinterpret_cast<uint16_t*>(slot_smem + oList);
+  double* const mu_acc = reinterpret_cast<double*>(slot_smem + oMu);
+  double* const th_acc = mu_acc + U;
 
   for (int q = tid; q < U; q += nthr) {
     const int pos = Rt > 1 ? (int)__umulhi((uint32_t)q, magic) : q;
-    sm.N[q] = t.N0 ? (uint32_t)__ldg(t.N0 + __ldg(t.rec + 3 * pos).x) : 0u;
+    slot_smem[oN + q] = t.N0 ? (uint32_t)__ldg(t.N0 + __ldg(t.rec + 3 * pos).x) : 0u;
   }
-  for (int k = tid; k < 4 * Rt; k += nthr) sm.racc[k] = 0;
+  for (int k = tid; k < t.ring * Rt; k += nthr) slot_smem[oR + (k / Rt) * ring_stride + t.E * Rt + k % Rt] = 0u;
+  for (int k = tid; k < 8 * Rt; k += nthr) slot_smem[oRacc + k] = 0u;
   for (int k = tid; k < 4 * U + t.n_ex * Rt; k += nthr) __stcg(acc + k, 0ull);
   if (GRAD) {
-    for (int q = tid; q < U; q += nthr) sm.mu_acc[q] = 0.0;
-    for (int k = tid; k < 3 * t.n_ex * Rt; k += nthr) sm.th_acc[k] = 0.0;
+    for (int q = tid; q < U; q += nthr) mu_acc[q] = 0.0;
+    for (int k = tid; k < 3 * t.n_ex * Rt; k += nthr) th_acc[k] = 0.0;
   }
   // ctr[0..1]: tasks handed out in phase 0 (by slot parity), ctr[2]: in phase
   // 1, ctr[4..6]: listed units (by slot mod 3).  Each is reset in a slot in
   // which no warp can still read its former value.
-  if (tid < 8) sm.ctr[tid] = tid < 3 ? nwarps : 0;
+  if (tid < 8) ctr[tid] = tid < 3 ? nwarps : 0;
   __threadfence();
   __syncthreads();
 
   const int last = SCHEME == 0 ? p.K + 1 : p.K + t.L - 1;
-  const int64_t ring_stride = (int64_t)t.E * Rt;
   int mod_ring = 0, mod3 = 0;
   const int ntask0 = (U + L - 1) / L;
   for (int slot = 1; slot <= last; ++slot) {
     mod_ring = mod_ring + 1 == t.ring ? 0 : mod_ring + 1;
     mod3 = mod3 == 2 ? 0 : mod3 + 1;
-    int* const count = sm.ctr + 4 + mod3;
+    int* const count = ctr + 4 + mod3;
     if (tid == 0) {
-      sm.ctr[(slot + 1) & 1] = nwarps;
-      sm.ctr[2] = nwarps;
-      sm.ctr[4 + (mod3 == 2 ? 0 : mod3 + 1)] = 0;
+      ctr[(slot + 1) & 1] = nwarps;
+      ctr[2] = nwarps;
+      ctr[4 + (mod3 == 2 ? 0 : mod3 + 1)] = 0;
     }
     int ntask = ntask0, listed = U;
 #pragma unroll 1
     for (int phase = 0; phase < 2; ++phase) {
-      int* const next = phase == 0 ? sm.ctr + (slot & 1) : sm.ctr + 2;
+      int* const next = phase == 0 ? ctr + (slot & 1) : ctr + 2;
 #pragma unroll 1
       for (int task = warp; task < ntask;) {
         const int idx = task * L + lane;
         bool act = lane < L && idx < listed;
         bool heavy = false, wait = phase == 1;  // x > m: listed, or drawn here
         int q = 0, r = 0;
-        int32_t i = 0, tau = 0, ec = -1, m = 0, e0 = 0, deg = 0;
+        int32_t i = 0, tau = 0, ec = -1, m = 0, e0 = 0, e1 = 0;
+        int ocur = oR;  // this step's routed counts
         uint32_t y = 0;
-        int32_t* rcur = sm.R;
         if (act) {
-          q = phase == 0 ? idx : sm.list[idx];
+          q = phase == 0 ? idx : list[idx];
           const int pos = Rt > 1 ? (int)__umulhi((uint32_t)q, magic) : q;
           r = q - pos * Rt;
-          const int4 ra = __ldg(t.rec + 3 * pos), rb = __ldg(t.rec + 3 * pos + 1);
+          const int4 ra = __ldg(t.rec + 3 * pos), rb = __ldg(t.rec + 3 * pos + 1), rc = __ldg(t.rec + 3 * pos + 2);
           i = ra.x;
           ec = ra.z;
           m = ra.w;
           e0 = rb.x;
-          deg = rb.y;
+          e1 = rb.y;
           if (SCHEME == 0) {
             tau = slot;
-            rcur = sm.R + (int64_t)(slot & 1) * ring_stride;
+            ocur = oR + (slot & 1) * ring_stride;
           } else {
             tau = slot - ra.y;
-            int rs = mod_ring - __ldg(t.rec + 3 * pos + 2).y;
-            rs = rs < 0 ? rs + t.ring : rs;
-            rcur = sm.R + (int64_t)rs * ring_stride;
+            const int rs = mod_ring - rc.y;
+            ocur = oR + (rs < 0 ? rs + t.ring : rs) * ring_stride;
             act = tau >= 1 && tau <= p.K;
           }
           const bool draws = tau <= p.K;
           if (EXT && p.mtab && act && draws) m = __ldg(p.mtab + (int64_t)(tau - 1) * n + i);
-          const uint32_t nprev = sm.N[q];
+          const uint32_t nprev = slot_smem[oN + q];
           y = nprev;
           if (act && phase == 0) {
             uint32_t A = 0;
@@ -186,7 +174,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
                 const float garr = (float)(int32_t)A / lam - 1.0f;
                 if (!isnan(garr)) {
                   const float* dl = p.dlam + ((int64_t)(tau - 1) * t.n_ex + ec) * 3;
-                  double* th = sm.th_acc + (ec * Rt + r) * 3;
+                  double* th = th_acc + (ec * Rt + r) * 3;
                   th[0] += (double)(garr * __ldg(dl + 0));
                   th[1] += (double)(garr * __ldg(dl + 1));
                   th[2] += (double)(garr * __ldg(dl + 2));
@@ -194,8 +182,17 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
               }
             }
             if (SCHEME == 1 ? draws : slot >= 2) {
-              const int32_t* rin = SCHEME == 1 ? rcur : sm.R + (int64_t)((slot - 1) & 1) * ring_stride;
-              y = slot_gather(t, rb.z, rb.w, rin, Rt, r, SCHEME == 1 ? nprev + A : nprev);
+              // sums held at kTop, beyond which the caller latches an overflow
+              constexpr uint32_t kTop = (uint32_t)kStateLimit + 1u;
+              const int oin = (SCHEME == 1 ? ocur : oR + ((slot - 1) & 1) * ring_stride) + r;
+              uint32_t in = (slot_smem[oin + rb.z * Rt] + slot_smem[oin + rb.w * Rt]) + slot_smem[oin + rc.x * Rt];
+              for (int32_t k = 0; k < rc.w; ++k) {
+                in = in < kTop ? in : kTop;
+                in += slot_smem[oin + __ldg(t.in_edge + rc.z + k) * Rt];
+              }
+              in = in < kTop ? in : kTop;
+              y = SCHEME == 1 ? nprev + A : nprev;
+              y = (y < kTop ? y : kTop) + in;
               if (y > (uint32_t)kStateLimit) {
                 cx.err |= kErrOverflow;
                 y = (uint32_t)kStateLimit;
@@ -212,10 +209,10 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
             act = draws && !heavy;
             // backward: the state less this step's departures, a listed unit's
             // A kept beside it (its x = y is the state without A)
-            if (SCHEME == 0 || heavy) sm.N[q] = y + (SCHEME == 0 ? A : 0u);
-            if (SCHEME == 0 && heavy && ec >= 0) sm.aex[ec * Rt + r] = (int32_t)A;
+            if (SCHEME == 0 || heavy) slot_smem[oN + q] = y + (SCHEME == 0 ? A : 0u);
+            if (SCHEME == 0 && heavy && ec >= 0) slot_smem[oAex + ec * Rt + r] = A;
           } else if (SCHEME == 0 && act && ec >= 0) {
-            y -= (uint32_t)sm.aex[ec * Rt + r];
+            y -= slot_smem[oAex + ec * Rt + r];
           }
         }
         if (phase == 0) {
@@ -224,7 +221,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
             int at = 0;
             if (lane == __ffs(hb) - 1) at = atomicAdd(count, __popc(hb));
             at = __shfl_sync(kFull, at, __ffs(hb) - 1);
-            if (heavy) sm.list[at + __popc(hb & ((1u << lane) - 1u))] = (uint16_t)q;
+            if (heavy) list[at + __popc(hb & ((1u << lane) - 1u))] = (uint16_t)q;
           }
         }
         if (act) {
@@ -254,12 +251,12 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
           // before, so the departure's are not live beside them; its sums and
           // the state are written after the loop (in its first pass they cost
           // 8%: 100-station DAG backward 351 against 329 ms).
-          int32_t e = e0, re = e0 * Rt + r, rem = 0;
-          const int32_t e1 = e0 + deg;
+          int32_t e = e0, rem = 0;
+          int orow = ocur + e0 * Rt + r;
           if (EXT && D >= 0) {
             base = -1;
             rem = nb = D;
-            if (deg > 0) bc = as_const(__ldg(t.qc + e));
+            if (e < e1) bc = as_const(__ldg(t.qc + e));
           }
 #pragma unroll 1
           while (base >= 0 || e < e1) {
@@ -272,23 +269,23 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
                 dep.branch = branch;
                 dep.T = T;
                 dep.p = pw;
-                sm.mu_acc[q] += (double)departure_score(dep, v, (int32_t)y, m, __ldg(t.mu + i), p.h, __ldg(p.p0f + i));
+                mu_acc[q] += (double)departure_score(dep, v, (int32_t)y, m, __ldg(t.mu + i), p.h, __ldg(p.p0f + i));
               }
               D = rem;
             } else {
-              rcur[re] = v;
+              slot_smem[orow] = (uint32_t)v;
               rem = rem - v;
               ++e;
-              re += Rt;
+              orow += Rt;
             }
             nb = rem;
             if (e < e1) bc = as_const(__ldg(t.qc + e));
           }
           if (SCHEME == 0) {
-            sm.N[q] -= (uint32_t)D;
+            slot_smem[oN + q] -= (uint32_t)D;
           } else {
             const uint32_t nn = y - (uint32_t)D;
-            sm.N[q] = nn;
+            slot_smem[oN + q] = nn;
             atomicAdd(acc + q, (unsigned long long)nn);
             if (nn > (uint32_t)m) slot_add(acc + U + q, nn - (uint32_t)m);
           }
@@ -321,7 +318,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
       const long long Q = (long long)__ldcg(acc + q), W = (long long)__ldcg(acc + U + q);
       const long long D = (long long)__ldcg(acc + 2 * (int64_t)U + q), X = (long long)__ldcg(acc + 3 * (int64_t)U + q);
       const long long A = ra.z >= 0 ? (long long)__ldcg(acc + 4 * (int64_t)U + ra.z * Rt + r) : 0;
-      unsigned long long* rr = reinterpret_cast<unsigned long long*>(sm.racc + 4 * r);
+      unsigned long long* rr = reinterpret_cast<unsigned long long*>(slot_smem + oRacc + 8 * r);
       atomicAdd(rr + 0, (unsigned long long)Q);
       atomicAdd(rr + 1, (unsigned long long)D);
       atomicAdd(rr + 2, (unsigned long long)X);
@@ -331,7 +328,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
       s[2] += D;
       s[3] += X;
       s[4] += A;
-      s[5] += (long long)sm.N[q];
+      s[5] += (long long)slot_smem[oN + q];
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
@@ -343,7 +340,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
   }
   __syncthreads();
   int64_t* const st_rep = p.stats + 5 * (int64_t)n + 4 * r0;
-  for (int k = tid; k < 4 * Rt; k += nthr) st_rep[k] = sm.racc[k];
+  for (int k = tid; k < 4 * Rt; k += nthr) st_rep[k] = reinterpret_cast<const long long*>(slot_smem + oRacc)[k];
   if (GRAD) {
     // S_r: mu_i sums, then (a, b, phase) summed over external stations in order
     const int64_t C = (int64_t)n + 3;
@@ -353,11 +350,11 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
       int64_t to;
       double v;
       if (c < n) {
-        v = sm.mu_acc[c * Rt + r];
+        v = mu_acc[c * Rt + r];
         to = __ldg(t.rec + 3 * c).x;
       } else {
         v = 0.0;
-        for (int32_t ec = 0; ec < t.n_ex; ++ec) v += sm.th_acc[(ec * Rt + r) * 3 + (c - n)];
+        for (int32_t ec = 0; ec < t.n_ex; ++ec) v += th_acc[(ec * Rt + r) * 3 + (c - n)];
         to = c;
       }
       p.scores[(r0 + r) * C + to] = v;
