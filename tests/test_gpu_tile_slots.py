@@ -79,3 +79,37 @@ def test_small_large_small_on_one_handle(Bd, orc, scheme):
             assert np.array_equal(got, want), R
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("scheme", [0, 1])
+@pytest.mark.parametrize("fan", [1, 3, 4, 9])
+def test_fan_in(Bd, orc, scheme, fan):
+    """A station with more in-edges than its record holds (three)."""
+    row_ptr, col, prob = W.csr_from_edges(fan + 1, [(i, fan, 0.9) for i in range(fan)])
+    arr = W.Arrivals(kind=W.ARR_SINUSOID, w=np.full(fan + 1, 9.0), a=1.0, b=0.2, period=5.0)
+    net = W.Network(fan + 1, row_ptr, col, prob, np.full(fan + 1, 4), np.full(fan + 1, 1.3), arr)
+    h = Bd.EulerNet(net)
+    try:
+        h.set_option(Bd.OPT_FORM, 1)
+        got = h.simulate(scheme, 0.1, 2.0, 40, 3).cpu().numpy()
+    finally:
+        h.close()
+    assert np.array_equal(got, orc.simulate(net, scheme, 0.1, 2.0, 40, 3)["stats"])
+
+
+def test_batch_of_both_schemes(Bd, orc):
+    """Both schemes in one batch run side by side, small tiles in place and
+    larger ones listed, and the batch runs again on the same plan."""
+    nets = [_net(n, 2, True, n % 2 == 0) for n in (1, 4, 9, 40, 41, 120)]
+    runs = [(j % 2, 0.1, 1.0 + 0.3 * j, R, 50 + j) for j, R in enumerate((7, 200, 33, 90, 64, 130))]
+    hs = [Bd.EulerNet(x) for x in nets]
+    b = Bd.Batch(hs, runs)
+    try:
+        for _ in range(2):
+            got = [s.cpu().numpy() for s in b.run()]
+            for net, r, g in zip(nets, runs, got):
+                assert np.array_equal(g, orc.simulate(net, r[0], r[1], r[2], r[3], r[4])["stats"]), r
+    finally:
+        b.close()
+        for h in hs:
+            h.close()
