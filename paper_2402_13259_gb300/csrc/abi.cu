@@ -134,6 +134,48 @@ void eulernet::step_lam(const euler_net& h, double dt, int64_t j0, int64_t cnt, 
   }
 }
 
+// The persistent form's per-unit sums for `grid` CTAs, into p.  Grown by
+// doubling and kept until the handle goes: a graph captured from an earlier
+// call may hold the former array, and a call may itself be under capture.
+static int slot_scratch(euler_net* h, int grid, int Rt, RunParams* p) {
+  p->acc_stride = slot_acc_len(h->n, h->n_ex, Rt);
+  const size_t need = (size_t)(p->acc_stride * grid);
+  if (need > h->tacc_cap) {
+    const size_t len = std::max(need, 2 * h->tacc_cap);
+    unsigned long long* a = nullptr;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+    cudaError_t e = cudaMalloc(&a, sizeof(unsigned long long) * len);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return cuda_fail(e, "per-unit sums");
+    if (h->d_tacc) h->tacc_old.push_back(h->d_tacc);
+    h->d_tacc = a;
+    h->tacc_cap = len;
+  }
+  p->acc = h->d_tacc;
+  return EULER_OK;
+}
+
+// The launches of a persistent-form run (see SlotPlan): p complete but for what
+// the plan decides.  One launch covers at most about 2e10 station-step updates
+// (about a second), a whole number of waves of tiles.
+int eulernet::run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp, int grid, cudaStream_t s) {
+  p.tile_reps = sp.Rt;
+  p.task_lanes = sp.lanes;
+  p.task_inline = sp.in_place;
+  const int rc = slot_scratch(h, grid, sp.Rt, &p);
+  if (rc) return rc;
+  const double wave = (double)h->n * (double)sp.Rt * (double)p.K * grid;
+  const int64_t step = (int64_t)grid * std::max<int64_t>(1, (int64_t)(2e10 / wave));
+  for (int64_t t0 = 0; t0 < sp.tiles; t0 += step) {
+    p.tile0 = t0;
+    p.num_tiles = std::min(sp.tiles, t0 + step);
+    const cudaError_t e = launch_persistent(h->tables(), p, mode, grid, sp.block, (int)sp.smem, s);
+    if (e != cudaSuccess) return cuda_fail(e, "persistent kernel launch");
+  }
+  return EULER_OK;
+}
+
 namespace {
 
 int refresh_step_tables(euler_net* h, double dt, double T, cudaStream_t s) {
@@ -183,48 +225,6 @@ int eulernet::prepare_step_tables(euler_net* h, double dt, double T, cudaStream_
   return refresh_step_tables(h, dt, T, s);
 }
 
-namespace {
-
-struct Plan {
-  int form = 1, tile_reps = 32, block = 32, grid = 1, lanes = 32;
-  bool in_place = false;
-  int64_t smem = 0, num_tiles = 0;
-  PipePlan pipe;
-};
-
-// Cut the level-ordered stations into W contiguous slices and record, per
-// slice, which other slices it receives from and sends to.
-bool make_pipe_plan(const euler_net* h, int W, PipePlan* pp) {
-  const int32_t n = h->n;
-  if (W < 1 || W > 32 || W > n) return false;
-  pp->W = W;
-  for (int w = 0; w <= W; ++w) pp->wbeg[w] = (int32_t)(((int64_t)w * n) / W);
-  std::vector<int32_t> owner(n, 0);
-  for (int w = 0; w < W; ++w)
-    for (int32_t k = pp->wbeg[w]; k < pp->wbeg[w + 1]; ++k) owner[h->lvl_station[k]] = w;
-  for (int w = 0; w < 32; ++w) pp->prod[w] = pp->cons[w] = 0u;
-  for (int32_t i = 0; i < n; ++i)
-    for (int32_t e = h->row_ptr[i]; e < h->row_ptr[i + 1]; ++e) {
-      const int a = owner[i], b = owner[h->col[e]];
-      if (a == b) continue;
-      if (a > b) return false;  // cannot happen for level order
-      pp->cons[a] |= 1u << b;
-      pp->prod[b] |= 1u << a;
-    }
-  return true;
-}
-
-// Launch shape of the persistent form (tile_slots.cuh) for R replications.
-struct SlotPlan {
-  int Rt = 0, block = 32, lanes = 32;
-  bool in_place = false;  // units with x > m drawn in place
-  int64_t smem = 0, tiles = 0;
-  double fill = 1.0;      // share of the SMs' replication slots in use
-};
-
-bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
-
-
 // One CTA of up to 1024 threads per SM: against two or four smaller ones per
 // SM (each with its own barriers and code position) the 100-station DAG ran
 // 147 and 165 ms instead of 137 (forward, 9,973 replications, 4,000 steps).
@@ -239,9 +239,10 @@ bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
 // 1.9 tasks 20.8 ms listed, 24.3 ms in place).
 //
 // Returns false if not even one replication fits a tile.
-bool plan_slots(const euler_net* h, int64_t R, bool grad, int force_Rt, int force_block, SlotPlan* sp) {
+bool eulernet::plan_slots(const euler_net* h, int64_t R, bool grad, int32_t soj, int force_Rt, int force_block,
+                          SlotPlan* sp) {
   const int32_t ring = h->tables().ring;
-  auto bytes = [&](int64_t Rt) { return slot_smem_bytes(h->n, h->E, ring, h->n_ex, Rt, grad); };
+  auto bytes = [&](int64_t Rt) { return slot_smem_bytes(h->n, h->E, ring, h->n_ex, Rt, grad, soj); };
   const int64_t limit = h->smem_optin;
   const int64_t per_rep = (bytes(33) - bytes(1)) / 32;
   int64_t Rmax = (limit - 256) / per_rep + 1;
@@ -285,9 +286,43 @@ bool plan_slots(const euler_net* h, int64_t R, bool grad, int force_Rt, int forc
 // whole GPU (n R >= 2^18) the tiles' coarseness decides: with every SM's
 // replication slots in use the persistent form is 1.1 (2,000 stations,
 // s = 10 .. 10,000) to 1.6 times (100 stations) as fast.
-bool hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp) {
+bool eulernet::hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp) {
   return (int64_t)h->n * R >= kHbmMinUnitsPerStep && sp.fill < kTileMinFill;
 }
+
+namespace {
+
+struct Plan {
+  int form = 1, tile_reps = 32, block = 32, grid = 1;
+  SlotPlan slots;
+  int64_t smem = 0, num_tiles = 0;
+  PipePlan pipe;
+};
+
+// Cut the level-ordered stations into W contiguous slices and record, per
+// slice, which other slices it receives from and sends to.
+bool make_pipe_plan(const euler_net* h, int W, PipePlan* pp) {
+  const int32_t n = h->n;
+  if (W < 1 || W > 32 || W > n) return false;
+  pp->W = W;
+  for (int w = 0; w <= W; ++w) pp->wbeg[w] = (int32_t)(((int64_t)w * n) / W);
+  std::vector<int32_t> owner(n, 0);
+  for (int w = 0; w < W; ++w)
+    for (int32_t k = pp->wbeg[w]; k < pp->wbeg[w + 1]; ++k) owner[h->lvl_station[k]] = w;
+  for (int w = 0; w < 32; ++w) pp->prod[w] = pp->cons[w] = 0u;
+  for (int32_t i = 0; i < n; ++i)
+    for (int32_t e = h->row_ptr[i]; e < h->row_ptr[i + 1]; ++e) {
+      const int a = owner[i], b = owner[h->col[e]];
+      if (a == b) continue;
+      if (a > b) return false;  // cannot happen for level order
+      pp->cons[a] |= 1u << b;
+      pp->prod[b] |= 1u << a;
+    }
+  return true;
+}
+
+bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
+
 
 int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
   const int64_t limit = h->smem_optin;
@@ -325,7 +360,7 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
   SlotPlan sp;
   if (pl->form == 1) {
     const int block = h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : 0;
-    const bool tiled = plan_slots(h, R, false, Rt, block, &sp);
+    const bool tiled = plan_slots(h, R, false, 0, Rt, block, &sp);
     if (!tiled && forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "network tile does not fit in shared memory");
     const bool large = forced_form <= 0 && (int64_t)h->n * R >= kHbmMinUnitsPerStep;
     const bool bad_block = block > 0 && (block % 32 || (Rt > 0 && block % Rt) || block > (large ? 256 : 512));
@@ -341,14 +376,13 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
     pl->num_tiles = (R + 31) / 32;
     return EULER_OK;
   }
+  pl->slots = sp;
   pl->tile_reps = sp.Rt;
   pl->block = sp.block;
-  pl->lanes = sp.lanes;
-  pl->in_place = sp.in_place;
   pl->smem = sp.smem;
   pl->num_tiles = sp.tiles;
   int per_sm = 0;
-  cudaError_t e = persistent_occupancy(scheme, pl->block, (int)pl->smem, &per_sm);
+  cudaError_t e = persistent_occupancy(kSlotPlain, scheme, pl->block, (int)pl->smem, &per_sm);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
   if (per_sm < 1) {
     if (forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "persistent kernel cannot be resident");
@@ -844,28 +878,6 @@ int euler_net_plan(euler_net* h, int32_t scheme, int64_t R, int32_t* form, int32
 
 namespace {
 
-// The persistent form's per-unit sums for `grid` CTAs, into p.  Grown by
-// doubling and kept until the handle goes: a graph captured from an earlier
-// call may hold the former array, and a call may itself be under capture.
-int slot_scratch(euler_net* h, int grid, int Rt, RunParams* p) {
-  p->acc_stride = slot_acc_len(h->n, h->n_ex, Rt);
-  const size_t need = (size_t)(p->acc_stride * grid);
-  if (need > h->tacc_cap) {
-    const size_t len = std::max(need, 2 * h->tacc_cap);
-    unsigned long long* a = nullptr;
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
-    cudaError_t e = cudaMalloc(&a, sizeof(unsigned long long) * len);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (e != cudaSuccess) return cuda_fail(e, "per-unit sums");
-    if (h->d_tacc) h->tacc_old.push_back(h->d_tacc);
-    h->d_tacc = a;
-    h->tacc_cap = len;
-  }
-  p->acc = h->d_tacc;
-  return EULER_OK;
-}
-
 template <class T>
 int grow(T** p, size_t* cap, size_t need) {
   if (need <= *cap && *p) return EULER_OK;
@@ -874,22 +886,6 @@ int grow(T** p, size_t* cap, size_t need) {
   CUDA_TRY(cudaMalloc(p, sizeof(T) * std::max<size_t>(need, 1)));
   *cap = need;
   return EULER_OK;
-}
-
-// One launch covers at most about 2e10 station-step updates (about a second),
-// a whole number of waves of tiles.
-template <class Launch>
-cudaError_t launch_tiles(const euler_net* h, RunParams p, int grid, Launch launch) {
-  const int64_t tiles = p.num_tiles;
-  const double wave = (double)h->n * (double)p.tile_reps * (double)p.K * grid;
-  const int64_t step = (int64_t)grid * std::max<int64_t>(1, (int64_t)(2e10 / wave));
-  cudaError_t e = cudaSuccess;
-  for (int64_t t0 = 0; t0 < tiles && e == cudaSuccess; t0 += step) {
-    p.tile0 = t0;
-    p.num_tiles = std::min(tiles, t0 + step);
-    e = launch(p);
-  }
-  return e;
 }
 
 // The run parameters of a plain simulation call (tables current for dt).
@@ -919,6 +915,7 @@ RunParams simulate_params(const euler_net* h, int32_t scheme, double dt, int64_t
   p.tile0 = 0;
   p.acc = nullptr;
   p.acc_stride = 0;
+  p.soj = SojournRun{};
   p.muh = h->d_muh;
   p.dep_mode = h->dep_mode();
   p.mtab = h->mtab();
@@ -969,15 +966,7 @@ int euler_net_simulate(euler_net* h, int32_t scheme, double dt, double T, int64_
     return EULER_OK;
   }
   if (pl.form == 1) {
-    p.task_lanes = pl.lanes;
-    p.task_inline = pl.in_place;
-    rc = slot_scratch(h, pl.grid, pl.tile_reps, &p);
-    if (rc) return rc;
-    cudaError_t e = launch_tiles(h, p, pl.grid, [&](const RunParams& pt) {
-      return launch_persistent(t, pt, pl.grid, pl.block, (int)pl.smem, s);
-    });
-    if (e != cudaSuccess) return cuda_fail(e, "persistent kernel launch");
-    return EULER_OK;
+    return run_slots(h, p, kSlotPlain, pl.slots, pl.grid, s);
   }
   return run_hbm_form(h, t, p, pl.block, s, HbmExtra());
 } catch (const std::bad_alloc&) {
@@ -1071,7 +1060,7 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   // station and replication in global memory, in the same step order).
   const int forced = (int)h->opt[EULER_OPT_FORM];
   SlotPlan sp;
-  const bool tiled = plan_slots(h, R, true, 0, 0, &sp);
+  const bool tiled = plan_slots(h, R, true, 0, 0, 0, &sp);
   if (forced == 2 || (forced <= 0 && (tiled ? hbm_beats_tiles(h, R, sp) : (int64_t)h->n * R >= kHbmMinUnitsPerStep))) {
     const int64_t ld = (R + 3) / 4 * 4;
     rc = grow(&h->d_gmu, &h->gmu_cap, (size_t)(h->n * ld));
@@ -1120,7 +1109,7 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   }
   if (!tiled) return fail(EULER_ERR_TOO_LARGE, "gradient tile does not fit in shared memory");
   int per_sm = 0;
-  cudaError_t e = grad_occupancy(scheme, sp.block, (int)sp.smem, &per_sm);
+  cudaError_t e = persistent_occupancy(kSlotGrad, scheme, sp.block, (int)sp.smem, &per_sm);
   if (e != cudaSuccess) return cuda_fail(e, "gradient occupancy query");
   if (per_sm < 1) return fail(EULER_ERR_TOO_LARGE, "gradient kernel cannot be resident");
   const int64_t tiles = sp.tiles;
@@ -1137,12 +1126,6 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   p.R = R;
   p.rep_begin = rep_begin;
   p.scheme = scheme;
-  p.tile_reps = sp.Rt;
-  p.num_tiles = tiles;
-  p.task_lanes = sp.lanes;
-  p.task_inline = sp.in_place;
-  rc = slot_scratch(h, grid, sp.Rt, &p);
-  if (rc) return rc;
   p.cap = h->opt[EULER_OPT_SAMPLER_CAP] > 0 ? (int32_t)h->opt[EULER_OPT_SAMPLER_CAP] : 1000;
   p.stats = stats;
   p.err = h->d_err;
@@ -1154,10 +1137,8 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   p.dep_mode = 0;
   p.mtab = h->mtab();
   CUDA_TRY(cudaMemsetAsync(stats, 0, sizeof(int64_t) * (size_t)euler_stats_len(h->n, R), s));
-  e = launch_tiles(h, p, grid, [&](const RunParams& pt) {
-    return launch_persistent_grad(h->tables(), pt, grid, sp.block, (int)sp.smem, s);
-  });
-  if (e != cudaSuccess) return cuda_fail(e, "gradient kernel launch");
+  rc = run_slots(h, p, kSlotGrad, sp, grid, s);
+  if (rc) return rc;
   e = launch_grad_reduce(h->n, R, dt, stats, scores, h->d_gpartial, grad, value, grad_var,
                                        h->opt[EULER_OPT_GRAD_CENTER] > 0, s);
   if (e != cudaSuccess) return cuda_fail(e, "gradient reduction launch");

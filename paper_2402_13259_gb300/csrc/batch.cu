@@ -101,7 +101,7 @@ int64_t pow2_floor(int64_t v) {
 
 // Shared memory of network j's tile of Rt replications.
 int64_t tile_bytes(const euler_net* h, int64_t Rt) {
-  return slot_smem_bytes(h->n, h->E, h->tables().ring, h->n_ex, Rt, false);
+  return slot_smem_bytes(h->n, h->E, h->tables().ring, h->n_ex, Rt, false, 0);
 }
 
 bool runs_hbm(const euler_batch* b, int j) { return b->is_hbm[j] != 0; }

@@ -158,6 +158,17 @@ struct HbmExtra {
 int run_hbm_form(euler_net* h, const NetTables& t, const RunParams& p, int block, cudaStream_t s,
                  const HbmExtra& x);
 
+// Launch shape of the persistent form (tile_slots.cuh) for R replications.
+struct SlotPlan {
+  int Rt = 0, block = 32, lanes = 32;
+  bool in_place = false;  // units with x > m drawn in place
+  int64_t smem = 0, tiles = 0;
+  double fill = 1.0;      // share of the SMs' replication slots in use
+};
+bool plan_slots(const euler_net* h, int64_t R, bool grad, int32_t soj, int force_Rt, int force_block, SlotPlan* sp);
+bool hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp);
+int run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp, int grid, cudaStream_t s);
+
 // A plain simulation call in the HBM form (the per-step kernels; the batched
 // form's large networks): tables made current for (dt, T), `block` threads
 // per step kernel, `graph_steps` slots per graph replay (0: default), at most

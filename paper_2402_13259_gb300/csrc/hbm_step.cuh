@@ -7,6 +7,7 @@
 
 #include "internal.h"
 #include "sampling.cuh"
+#include "sojourn_step.cuh"
 #include "unit.cuh"
 
 namespace eulernet {
@@ -68,33 +69,6 @@ __device__ __forceinline__ void hbm_add_scores(const NetTables& t, const RunPara
 // station's warp may read the word while it is rewritten in the same launch:
 // it then sees either a different station or a due step it is not
 // processing, so the 64-bit word is read and written whole.
-constexpr unsigned long long kSojDone = 0xFFFFFFFFull << 32;
-
-__device__ __forceinline__ unsigned long long soj_pack(int32_t station, int32_t due, bool setup) {
-  return ((unsigned long long)(uint32_t)station << 32) | ((unsigned long long)(uint32_t)due << 1) |
-         (setup ? 1ull : 0ull);
-}
-
-// b^k (k >= 0) by binary powering, multiplications in a fixed order.
-__device__ __forceinline__ float soj_pow_int(float b, int32_t k) {
-  float r = 1.0f;
-  while (k > 0) {
-    if (k & 1) r = r * b;
-    b = b * b;
-    k >>= 1;
-  }
-  return r;
-}
-
-// Lemma 3: P(the tagged customer's service continues through the step | the
-// step's departure draw had input x and output d > 0, m servers).
-__device__ __forceinline__ float soj_stay(int32_t x, int32_t d, int32_t m) {
-  if (x <= m) return (float)(x - d) / (float)x;
-  const float q = (float)(m - 1) / (float)m;
-  if (x <= m + d) return soj_pow_int(q, x - m) * ((float)(x - d) / (float)m);
-  return soj_pow_int(q, d);
-}
-
 // Setup of customer word *lp at station i after step tau (N = N_tau,i).
 template <bool EXT>
 __device__ __forceinline__ void soj_setup(const NetTables& t, const RunParams& p, const HbmState& hs,

@@ -35,6 +35,15 @@ struct NetTables {
                                // max(2, largest level gap of an edge + 1)
 };
 
+// Sojourn times (Algorithm 4): S tagged customers per replication enter
+// `station` in step tau0; out[r][c] is customer c's sojourn in steps, or minus
+// the steps accounted if it is still in the network at the end.
+struct SojournRun {
+  const int32_t* col;  // [E] destination station of each edge
+  int32_t* out;        // [R][S]
+  int32_t station, tau0, S;
+};
+
 // Per-call parameters.
 struct RunParams {
   const float4* p0;  // [n] BinomConst of 1 - e^{-mu_i dt}
@@ -56,6 +65,7 @@ struct RunParams {
   int32_t task_inline;     // persistent form: nonzero = units with x > m drawn in place, not listed
   unsigned long long* acc; // persistent form: per-unit sums, acc_stride entries per CTA
   int64_t acc_stride;
+  SojournRun soj;          // persistent form, sojourn kernels only
   const float* muh;      // [n] mu_i dt rounded to float (Eq. (1)/(2) departures)
   int32_t dep_mode;      // 0 exact (Algorithm 1), 1 Eq. (1), 2 Eq. (2)
   const int32_t* mtab;   // [K][n] servers per step (staffing schedule), or nullptr
@@ -78,14 +88,11 @@ inline void set_round_keys(uint32_t* rk, uint32_t key0, uint32_t key1) {
   }
 }
 
-// Shared-memory bytes of the step-by-step tile kernel (sojourn times) for a
-// tile of `tile_reps` with `ring` slots of routed counts.
-int64_t persistent_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t tile_reps);
-
 // Shared-memory bytes of the persistent kernel (tile_slots.cuh) for a tile of
-// Rt replications, and its per-unit sums (64-bit entries of global scratch per
+// Rt replications (with score sums if grad, with `soj` tagged customers per
+// replication), and its per-unit sums (64-bit entries of global scratch per
 // CTA).
-int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad);
+int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad, int32_t soj);
 inline int64_t slot_acc_len(int32_t n, int32_t n_ex, int64_t Rt) { return (4 * (int64_t)n + n_ex) * Rt; }
 // Whether `warps` warps draw the units with x > m of a slot of `tasks` tasks in
 // place instead of listing them (see plan_slots).
@@ -98,11 +105,7 @@ cudaError_t launch_batch(int scheme, bool ext, const NetTables* nets, const RunP
                          int num_items, int* next_item, unsigned long long* acc_scratch,
                          int64_t acc_slot_len, int grid, int block, int smem, cudaStream_t s);
 
-// Gradient form of the persistent kernel (scores into p.scores) and the
-// fixed-order reduction of L_m(r) S_r over replications.
-cudaError_t grad_occupancy(int scheme, int block, int smem, int* blocks_per_sm);
-cudaError_t launch_persistent_grad(const NetTables& t, const RunParams& p, int grid, int block,
-                                   int smem, cudaStream_t s);
+// Fixed-order reduction of L_m(r) S_r over replications.
 cudaError_t launch_grad_reduce(int32_t n, int64_t R, double dt, const int64_t* stats,
                                const double* scores, double* partial, double* grad, double* value,
                                double* grad_var, bool center, cudaStream_t s);
@@ -111,12 +114,14 @@ cudaError_t launch_grad_reduce(int32_t n, int64_t R, double dt, const int64_t* s
 cudaError_t launch_average(const int64_t* b, const int64_t* f, double* out, int64_t len,
                            cudaStream_t s);
 
-// Launch the persistent shared-memory kernel.
-cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int grid, int block,
+// The persistent shared-memory kernel: plain, with score sums (scores into
+// p.scores), or with tagged customers (p.soj).
+enum SlotMode { kSlotPlain = 0, kSlotGrad = 1, kSlotSojourn = 2 };
+cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int mode, int grid, int block,
                               int smem, cudaStream_t s);
 
 // Blocks of `block` threads with `smem` bytes that fit on one SM.
-cudaError_t persistent_occupancy(int scheme, int block, int smem, int* blocks_per_sm);
+cudaError_t persistent_occupancy(int mode, int scheme, int block, int smem, int* blocks_per_sm);
 
 // Level-pipelined form: W warps per 32-replication tile, warp w owns the
 // level-ordered station slice lvl_station[wbeg[w] .. wbeg[w+1]); prod[w] and

@@ -29,7 +29,7 @@ namespace eulernet {
 namespace {
 
 // Single network: CTAs loop over the tiles.
-template <int SCHEME, bool GRAD = false, bool EXT = true>
+template <int SCHEME, int MODE, bool EXT>
 __global__ void __launch_bounds__(kSlotThreads, 1)
     persistent_kernel(const __grid_constant__ NetTables t, const __grid_constant__ RunParams p) {
   float* rinv = reinterpret_cast<float*>(slot_smem);
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kSlotThreads, 1)
   SamplerCtx cx{rinv, p.cap, 0u};
   unsigned long long* const acc = p.acc + (int64_t)blockIdx.x * p.acc_stride;
   for (int64_t tile = p.tile0 + blockIdx.x; tile < p.num_tiles; tile += gridDim.x)
-    tile_slots<SCHEME, GRAD, EXT>(t, p, tile, acc, cx, p.rk);
+    tile_slots<SCHEME, MODE == kSlotGrad, EXT, MODE == kSlotSojourn>(t, p, tile, acc, cx, p.rk);
   latch(p.err, cx.err);
 }
 
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kSlotThreads, 1)
       reinterpret_cast<uint32_t*>(p_raw)[k] = reinterpret_cast<const uint32_t*>(runs + wi.x)[k];
     __syncthreads();
     cx.cap = p.cap;
-    tile_slots<SCHEME, false, EXT>(t, p, wi.y, acc, cx, p.rk);  // ends with a block barrier
+    tile_slots<SCHEME, false, EXT, false>(t, p, wi.y, acc, cx, p.rk);  // ends with a block barrier
     latch(p.err, cx.err);
     cx.err = 0;
     __syncthreads();  // t, p and s_item are rewritten next
@@ -195,26 +195,28 @@ __global__ void hbm_finish_kernel(NetTables t, RunParams p, HbmState hs, int64_t
 
 }  // namespace
 
-int64_t persistent_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t tile_reps) {
-  return 256 + 6 * 8 * (int64_t)n + 4 * 8 * (int64_t)tile_reps +
-         4 * ((int64_t)n + (int64_t)ring * E) * tile_reps;
-}
-
-int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad) {
+int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_t Rt, bool grad, int32_t soj) {
   int64_t words = 80 + Rt * (8 + (int64_t)n + (int64_t)ring * (E + 1) + n_ex) + (n * Rt + 1) / 2;
   words = (words + 3) / 4 * 4;
   if (grad) words += 2 * Rt * ((int64_t)n + 3 * (int64_t)n_ex);
+  words += 4 * Rt * (int64_t)soj;
   return 4 * words;
 }
 
 namespace {
 bool uses_ext(const RunParams& p) { return p.mtab != nullptr || p.dep_mode != 0; }
 
-template <bool GRAD>
+template <int MODE>
 const void* persistent_fn(int scheme, bool ext) {
   if (scheme == 0)
-    return ext ? (const void*)persistent_kernel<0, GRAD, true> : (const void*)persistent_kernel<0, GRAD, false>;
-  return ext ? (const void*)persistent_kernel<1, GRAD, true> : (const void*)persistent_kernel<1, GRAD, false>;
+    return ext ? (const void*)persistent_kernel<0, MODE, true> : (const void*)persistent_kernel<0, MODE, false>;
+  return ext ? (const void*)persistent_kernel<1, MODE, true> : (const void*)persistent_kernel<1, MODE, false>;
+}
+
+const void* persistent_fn(int mode, int scheme, bool ext) {
+  return mode == kSlotGrad      ? persistent_fn<kSlotGrad>(scheme, ext)
+         : mode == kSlotSojourn ? persistent_fn<kSlotSojourn>(scheme, ext)
+                                : persistent_fn<kSlotPlain>(scheme, ext);
 }
 
 const void* batch_fn(int scheme, bool ext) {
@@ -243,17 +245,17 @@ cudaError_t launch_fn(const void* fn, void** args, int grid, int block, int smem
 }
 }  // namespace
 
-cudaError_t persistent_occupancy(int scheme, int block, int smem, int* blocks_per_sm) {
-  const void* fns[2] = {persistent_fn<false>(scheme, false), persistent_fn<false>(scheme, true)};
+cudaError_t persistent_occupancy(int mode, int scheme, int block, int smem, int* blocks_per_sm) {
+  const void* fns[2] = {persistent_fn(mode, scheme, false), persistent_fn(mode, scheme, true)};
   return min_occupancy(fns, 2, block, smem, blocks_per_sm);
 }
 
-cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int grid, int block, int smem,
+cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int mode, int grid, int block, int smem,
                               cudaStream_t s) {
   NetTables tt = t;
   RunParams pp = p;
   void* args[] = {&tt, &pp};
-  return launch_fn(persistent_fn<false>(p.scheme, uses_ext(p)), args, grid, block, smem, s);
+  return launch_fn(persistent_fn(mode, p.scheme, uses_ext(p)), args, grid, block, smem, s);
 }
 
 cudaError_t batch_occupancy(int block, int smem, int* blocks_per_sm) {
@@ -266,19 +268,6 @@ cudaError_t launch_batch(int scheme, bool ext, const NetTables* nets, const RunP
                          int64_t acc_slot_len, int grid, int block, int smem, cudaStream_t s) {
   void* args[] = {&nets, &runs, &items, &num_items, &next_item, &acc_scratch, &acc_slot_len};
   return launch_fn(batch_fn(scheme, ext), args, grid, block, smem, s);
-}
-
-cudaError_t grad_occupancy(int scheme, int block, int smem, int* blocks_per_sm) {
-  const void* fns[2] = {persistent_fn<true>(scheme, false), persistent_fn<true>(scheme, true)};
-  return min_occupancy(fns, 2, block, smem, blocks_per_sm);
-}
-
-cudaError_t launch_persistent_grad(const NetTables& t, const RunParams& p, int grid, int block,
-                                   int smem, cudaStream_t s) {
-  NetTables tt = t;
-  RunParams pp = p;
-  void* args[] = {&tt, &pp};
-  return launch_fn(persistent_fn<true>(p.scheme, uses_ext(p)), args, grid, block, smem, s);
 }
 
 cudaError_t launch_grad_reduce(int32_t n, int64_t R, double dt, const int64_t* stats,
