@@ -170,7 +170,7 @@ int eulernet::run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp,
   for (int64_t t0 = 0; t0 < sp.tiles; t0 += step) {
     p.tile0 = t0;
     p.num_tiles = std::min(sp.tiles, t0 + step);
-    const cudaError_t e = launch_persistent(h->tables(), p, mode, grid, sp.block, (int)sp.smem, s);
+    const cudaError_t e = launch_persistent(h->tables(), p, mode, sp.resident, grid, sp.block, (int)sp.smem, s);
     if (e != cudaSuccess) return cuda_fail(e, "persistent kernel launch");
   }
   return EULER_OK;
@@ -276,6 +276,7 @@ bool eulernet::plan_slots(const euler_net* h, int64_t R, bool grad, int32_t soj,
   sp->lanes = (int)L;
   sp->block = force_block > 0 ? force_block : (int)(32 * std::max<int64_t>(1, std::min<int64_t>(kSlotThreads / 32, tasks)));
   sp->in_place = draws_in_place(tasks, sp->block / 32);
+  sp->resident = tasks <= sp->block / 32 && soj == 0 && (!grad || sp->block <= kSlotResGradThreads);
   sp->fill = (double)R / (double)(Rt * SM * waves_of(Rt));
   return true;
 }
@@ -382,7 +383,7 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
   pl->smem = sp.smem;
   pl->num_tiles = sp.tiles;
   int per_sm = 0;
-  cudaError_t e = persistent_occupancy(kSlotPlain, scheme, pl->block, (int)pl->smem, &per_sm);
+  cudaError_t e = persistent_occupancy(kSlotPlain, scheme, sp.resident, pl->block, (int)pl->smem, &per_sm);
   if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
   if (per_sm < 1) {
     if (forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "persistent kernel cannot be resident");
@@ -1109,7 +1110,7 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   }
   if (!tiled) return fail(EULER_ERR_TOO_LARGE, "gradient tile does not fit in shared memory");
   int per_sm = 0;
-  cudaError_t e = persistent_occupancy(kSlotGrad, scheme, sp.block, (int)sp.smem, &per_sm);
+  cudaError_t e = persistent_occupancy(kSlotGrad, scheme, sp.resident, sp.block, (int)sp.smem, &per_sm);
   if (e != cudaSuccess) return cuda_fail(e, "gradient occupancy query");
   if (per_sm < 1) return fail(EULER_ERR_TOO_LARGE, "gradient kernel cannot be resident");
   const int64_t tiles = sp.tiles;

@@ -162,6 +162,7 @@ int run_hbm_form(euler_net* h, const NetTables& t, const RunParams& p, int block
 struct SlotPlan {
   int Rt = 0, block = 32, lanes = 32;
   bool in_place = false;  // units with x > m drawn in place
+  bool resident = false;  // and no more tasks than warps: the kernel's RES variant
   int64_t smem = 0, tiles = 0;
   double fill = 1.0;      // share of the SMs' replication slots in use
 };

@@ -98,6 +98,7 @@ inline int64_t slot_acc_len(int32_t n, int32_t n_ex, int64_t Rt) { return (4 * (
 // place instead of listing them (see plan_slots).
 inline bool draws_in_place(int64_t tasks, int64_t warps) { return 2 * tasks <= 3 * warps; }
 constexpr int kSlotThreads = 1024;  // most threads per block (the register budget: 64)
+constexpr int kSlotResGradThreads = 512;  // of the resident gradient variant
 
 // Batched form: one persistent launch over (network, tile) work items.
 cudaError_t batch_occupancy(int block, int smem, int* blocks_per_sm);
@@ -115,13 +116,14 @@ cudaError_t launch_average(const int64_t* b, const int64_t* f, double* out, int6
                            cudaStream_t s);
 
 // The persistent shared-memory kernel: plain, with score sums (scores into
-// p.scores), or with tagged customers (p.soj).
+// p.scores), or with tagged customers (p.soj); `resident`: its RES variant
+// (plain and score sums only), see tile_slots.
 enum SlotMode { kSlotPlain = 0, kSlotGrad = 1, kSlotSojourn = 2 };
-cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int mode, int grid, int block,
-                              int smem, cudaStream_t s);
+cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int mode, bool resident, int grid,
+                              int block, int smem, cudaStream_t s);
 
 // Blocks of `block` threads with `smem` bytes that fit on one SM.
-cudaError_t persistent_occupancy(int mode, int scheme, int block, int smem, int* blocks_per_sm);
+cudaError_t persistent_occupancy(int mode, int scheme, bool resident, int block, int smem, int* blocks_per_sm);
 
 // Level-pipelined form: W warps per 32-replication tile, warp w owns the
 // level-ordered station slice lvl_station[wbeg[w] .. wbeg[w+1]); prod[w] and

@@ -29,15 +29,18 @@ namespace eulernet {
 namespace {
 
 // Single network: CTAs loop over the tiles.
-template <int SCHEME, int MODE, bool EXT>
-__global__ void __launch_bounds__(kSlotThreads, 1)
+// The resident gradient variant has no spills at 512 threads' registers (grad of
+// the tandem 8.7 -> 7.9 ms); the plain one is the faster at 1,024 threads' (5.0
+// against 5.8 ms forward), and covers tiles of up to 1,024 units there.
+template <int SCHEME, int MODE, bool EXT, bool RES>
+__global__ void __launch_bounds__(RES && MODE == kSlotGrad ? kSlotResGradThreads : kSlotThreads, 1)
     persistent_kernel(const __grid_constant__ NetTables t, const __grid_constant__ RunParams p) {
   float* rinv = reinterpret_cast<float*>(slot_smem);
   fill_rinv(rinv);
   SamplerCtx cx{rinv, p.cap, 0u};
   unsigned long long* const acc = p.acc + (int64_t)blockIdx.x * p.acc_stride;
   for (int64_t tile = p.tile0 + blockIdx.x; tile < p.num_tiles; tile += gridDim.x)
-    tile_slots<SCHEME, MODE == kSlotGrad, EXT, MODE == kSlotSojourn>(t, p, tile, acc, cx, p.rk);
+    tile_slots<SCHEME, MODE == kSlotGrad, EXT, MODE == kSlotSojourn, RES>(t, p, tile, acc, cx, p.rk);
   latch(p.err, cx.err);
 }
 
@@ -132,7 +135,7 @@ __global__ void __launch_bounds__(kSlotThreads, 1)
       reinterpret_cast<uint32_t*>(p_raw)[k] = reinterpret_cast<const uint32_t*>(runs + wi.x)[k];
     __syncthreads();
     cx.cap = p.cap;
-    tile_slots<SCHEME, false, EXT, false>(t, p, wi.y, acc, cx, p.rk);  // ends with a block barrier
+    tile_slots<SCHEME, false, EXT, false, false>(t, p, wi.y, acc, cx, p.rk);  // ends with a block barrier
     latch(p.err, cx.err);
     cx.err = 0;
     __syncthreads();  // t, p and s_item are rewritten next
@@ -206,17 +209,17 @@ int64_t slot_smem_bytes(int32_t n, int32_t E, int32_t ring, int32_t n_ex, int64_
 namespace {
 bool uses_ext(const RunParams& p) { return p.mtab != nullptr || p.dep_mode != 0; }
 
-template <int MODE>
+template <int MODE, bool RES>
 const void* persistent_fn(int scheme, bool ext) {
   if (scheme == 0)
-    return ext ? (const void*)persistent_kernel<0, MODE, true> : (const void*)persistent_kernel<0, MODE, false>;
-  return ext ? (const void*)persistent_kernel<1, MODE, true> : (const void*)persistent_kernel<1, MODE, false>;
+    return ext ? (const void*)persistent_kernel<0, MODE, true, RES> : (const void*)persistent_kernel<0, MODE, false, RES>;
+  return ext ? (const void*)persistent_kernel<1, MODE, true, RES> : (const void*)persistent_kernel<1, MODE, false, RES>;
 }
 
-const void* persistent_fn(int mode, int scheme, bool ext) {
-  return mode == kSlotGrad      ? persistent_fn<kSlotGrad>(scheme, ext)
-         : mode == kSlotSojourn ? persistent_fn<kSlotSojourn>(scheme, ext)
-                                : persistent_fn<kSlotPlain>(scheme, ext);
+const void* persistent_fn(int mode, int scheme, bool ext, bool resident) {
+  if (mode == kSlotSojourn) return persistent_fn<kSlotSojourn, false>(scheme, ext);
+  if (mode == kSlotGrad) return resident ? persistent_fn<kSlotGrad, true>(scheme, ext) : persistent_fn<kSlotGrad, false>(scheme, ext);
+  return resident ? persistent_fn<kSlotPlain, true>(scheme, ext) : persistent_fn<kSlotPlain, false>(scheme, ext);
 }
 
 const void* batch_fn(int scheme, bool ext) {
@@ -245,17 +248,17 @@ cudaError_t launch_fn(const void* fn, void** args, int grid, int block, int smem
 }
 }  // namespace
 
-cudaError_t persistent_occupancy(int mode, int scheme, int block, int smem, int* blocks_per_sm) {
-  const void* fns[2] = {persistent_fn(mode, scheme, false), persistent_fn(mode, scheme, true)};
+cudaError_t persistent_occupancy(int mode, int scheme, bool resident, int block, int smem, int* blocks_per_sm) {
+  const void* fns[2] = {persistent_fn(mode, scheme, false, resident), persistent_fn(mode, scheme, true, resident)};
   return min_occupancy(fns, 2, block, smem, blocks_per_sm);
 }
 
-cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int mode, int grid, int block, int smem,
-                              cudaStream_t s) {
+cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int mode, bool resident, int grid, int block,
+                              int smem, cudaStream_t s) {
   NetTables tt = t;
   RunParams pp = p;
   void* args[] = {&tt, &pp};
-  return launch_fn(persistent_fn(mode, p.scheme, uses_ext(p)), args, grid, block, smem, s);
+  return launch_fn(persistent_fn(mode, p.scheme, uses_ext(p), resident), args, grid, block, smem, s);
 }
 
 cudaError_t batch_occupancy(int block, int smem, int* blocks_per_sm) {

@@ -84,7 +84,14 @@ __device__ __forceinline__ void slot_add(unsigned long long* a, uint32_t v) {
 // 100-station DAG, 10,000 replications, 4 customers each, 2,000 steps: 118 ms
 // in the per-step kernels -> 65 ms; 162 stations, 102 replications, one step
 // at a time with a barrier after each level 161 -> 18 ms for 3,220 steps.
-template <int SCHEME, bool GRAD, bool EXT, bool SOJ>
+//
+// RES: each warp draws one and the same task in every slot (all units in place,
+// no more tasks than warps), so its units' records and states stay in
+// registers and a slot has no queue and no list.  Such runs are bound by the
+// latency of one unit's draws, 2 to 3 us a slot (three-station tandem, 1,000
+// replications, 2,402 slots 6.3 -> 5.0 ms; 100 stations, 1,237 replications,
+// both schemes 43 -> 40 ms).
+template <int SCHEME, bool GRAD, bool EXT, bool SOJ, bool RES>
 __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& p, int64_t tile,
                                            unsigned long long* const acc, SamplerCtx& cx,
                                            const uint32_t* rk) {
@@ -142,33 +149,45 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
   const int last = SCHEME == 0 ? p.K + 1 : p.K + t.L - 1;
   int mod_ring = 0, mod3 = 0;
   const int ntask0 = (U + L - 1) / L;
+  int4 ra = make_int4(0, 0, -1, 0), rb = make_int4(0, 0, 0, 0), rc = rb;
+  int q = 0, r = 0;
+  auto load_unit = [&](int unit) {
+    q = unit;
+    const int pos = Rt > 1 ? (int)__umulhi((uint32_t)q, magic) : q;
+    r = q - pos * Rt;
+    ra = __ldg(t.rec + 3 * pos);
+    rb = __ldg(t.rec + 3 * pos + 1);
+    rc = __ldg(t.rec + 3 * pos + 2);
+  };
+  const bool own = RES && lane < L && warp * L + lane < U;
+  uint32_t nres = 0;  // RES: the unit's state
+  if (own) {
+    load_unit(warp * L + lane);
+    nres = slot_smem[oN + q];
+  }
   for (int slot = 1; slot <= last; ++slot) {
     mod_ring = mod_ring + 1 == t.ring ? 0 : mod_ring + 1;
     mod3 = mod3 == 2 ? 0 : mod3 + 1;
     int* const count = ctr + 4 + mod3;
-    if (tid == 0) {
+    if (!RES && tid == 0) {
       ctr[(slot + 1) & 1] = nwarps;
       ctr[2] = nwarps;
       ctr[4 + (mod3 == 2 ? 0 : mod3 + 1)] = 0;
     }
     int ntask = ntask0, listed = U;
 #pragma unroll 1
-    for (int phase = 0; phase < 2; ++phase) {
+    for (int phase = 0; phase < (RES ? 1 : 2); ++phase) {
       int* const next = phase == 0 ? ctr + (slot & 1) : ctr + 2;
 #pragma unroll 1
       for (int task = warp; task < ntask;) {
         const int idx = task * L + lane;
-        bool act = lane < L && idx < listed;
+        bool act = RES ? own : lane < L && idx < listed;
         bool heavy = false, wait = phase == 1;  // x > m: listed, or drawn here
-        int q = 0, r = 0;
         int32_t i = 0, tau = 0, ec = -1, m = 0, e0 = 0, e1 = 0;
         int ocur = oR;  // this step's routed counts
         uint32_t y = 0;
         if (act) {
-          q = phase == 0 ? idx : list[idx];
-          const int pos = Rt > 1 ? (int)__umulhi((uint32_t)q, magic) : q;
-          r = q - pos * Rt;
-          const int4 ra = __ldg(t.rec + 3 * pos), rb = __ldg(t.rec + 3 * pos + 1), rc = __ldg(t.rec + 3 * pos + 2);
+          if (!RES) load_unit(phase == 0 ? idx : list[idx]);
           i = ra.x;
           ec = ra.z;
           m = ra.w;
@@ -185,7 +204,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
           }
           const bool draws = tau <= p.K;
           if (EXT && p.mtab && act && draws) m = __ldg(p.mtab + (int64_t)(tau - 1) * n + i);
-          const uint32_t nprev = slot_smem[oN + q];
+          const uint32_t nprev = RES ? nres : slot_smem[oN + q];
           y = nprev;
           if (act && phase == 0) {
             uint32_t A = 0;
@@ -230,8 +249,8 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
               if (y > (uint32_t)mp) slot_add(acc + U + q, y - (uint32_t)mp);
             }
             heavy = draws && (!EXT || p.dep_mode == 0) && y > (uint32_t)m;
-            wait = heavy && p.task_inline != 0;
-            heavy = heavy && p.task_inline == 0;
+            wait = heavy && (RES || p.task_inline != 0);
+            heavy = heavy && !wait;
             act = draws && !heavy;
             if (SOJ && SCHEME == 0 && !draws)  // slot K+1: the last setups
               for (int ci = r; ci < S * Rt; ci += Rt)
@@ -241,13 +260,16 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
                 }
             // backward: the state less this step's departures, a listed unit's
             // A kept beside it (its x = y is the state without A)
-            if (SCHEME == 0 || heavy) slot_smem[oN + q] = y + (SCHEME == 0 ? A : 0u);
+            if (RES)
+              nres = y + (SCHEME == 0 ? A : 0u);
+            else if (SCHEME == 0 || heavy)
+              slot_smem[oN + q] = y + (SCHEME == 0 ? A : 0u);
             if (SCHEME == 0 && heavy && ec >= 0) slot_smem[oAex + ec * Rt + r] = A;
           } else if (SCHEME == 0 && act && ec >= 0) {
             y -= slot_smem[oAex + ec * Rt + r];
           }
         }
-        if (phase == 0) {
+        if (!RES && phase == 0) {
           const unsigned hb = __ballot_sync(kFull, heavy);
           if (hb) {
             int at = 0;
@@ -314,10 +336,16 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
             if (e < e1) bc = as_const(__ldg(t.qc + e));
           }
           if (SCHEME == 0) {
-            slot_smem[oN + q] -= (uint32_t)D;
+            if (RES)
+              nres -= (uint32_t)D;
+            else
+              slot_smem[oN + q] -= (uint32_t)D;
           } else {
             const uint32_t nn = y - (uint32_t)D;
-            slot_smem[oN + q] = nn;
+            if (RES)
+              nres = nn;
+            else
+              slot_smem[oN + q] = nn;
             atomicAdd(acc + q, (unsigned long long)nn);
             if (nn > (uint32_t)m) slot_add(acc + U + q, nn - (uint32_t)m);
           }
@@ -362,12 +390,12 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
           atomicAdd(acc + 2 * (int64_t)U + q, (unsigned long long)(uint32_t)D);
           slot_add(acc + 3 * (int64_t)U + q, (uint32_t)rem);
         }
-        if (ntask <= nwarps) break;
+        if (RES || ntask <= nwarps) break;
         if (lane == 0) task = atomicAdd(next, 1);
         task = __shfl_sync(kFull, task, 0);
       }
       __syncthreads();
-      if (phase == 0) {
+      if (!RES && phase == 0) {
         listed = *count;
         if (listed == 0) break;  // uniform
         ntask = (listed + L - 1) / L;
@@ -375,6 +403,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
     }
   }
 
+  if (own) slot_smem[oN + q] = nres;
   // The tile's sums: over replications to the stations, over stations to the
   // replications; N_K from the state.
   __threadfence();
