@@ -17,6 +17,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -54,15 +55,41 @@ int cuda_fail(cudaError_t e, const char* where) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #expr); \
   } while (0)
 
-template <class T>
-cudaError_t upload(T** dst, const std::vector<T>& src, int64_t* counter) {
-  *dst = nullptr;
-  *counter += (int64_t)(src.size() * sizeof(T));
-  const size_t bytes = std::max<size_t>(src.size(), 1) * sizeof(T);
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(dst), bytes);
-  if (e != cudaSuccess) return e;
-  if (!src.empty()) e = cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
-  return e;
+// A handle's immutable tables in one device allocation, filled by one copy: a
+// dozen of each made most of euler_net_create's time (183 us for the
+// three-station tandem).
+struct TableImage {
+  std::vector<unsigned char> bytes;
+  std::vector<std::pair<void**, size_t>> at;  // pointer to set, offset
+  int64_t payload = 0;
+
+  template <class T>
+  void add(T** dst, const std::vector<T>& src) {
+    const size_t off = (bytes.size() + 255) / 256 * 256;
+    bytes.resize(off + std::max<size_t>(src.size(), 1) * sizeof(T));
+    if (!src.empty()) std::memcpy(bytes.data() + off, src.data(), src.size() * sizeof(T));
+    at.emplace_back(reinterpret_cast<void**>(dst), off);
+    payload += (int64_t)(src.size() * sizeof(T));
+  }
+
+  cudaError_t upload(void** base) {
+    cudaError_t e = cudaMalloc(base, bytes.size());
+    if (e != cudaSuccess) return e;
+    for (auto& pr : at) *pr.first = static_cast<unsigned char*>(*base) + pr.second;
+    return cudaMemcpy(*base, bytes.data(), bytes.size(), cudaMemcpyHostToDevice);
+  }
+};
+
+}  // namespace
+
+namespace {
+
+double sin_omega(const euler_net& h) { return 6.283185307179586 / h.period; }
+
+// The sinusoid's integral over (t0, t1], c0 and c1 the cosines at its ends.
+double sin_mean(const euler_net& h, int32_t i, double t0, double t1, double om, double c0, double c1) {
+  const double lam = h.w[i] * h.a * ((t1 - t0) + h.b * (c0 - c1) / om);
+  return lam > 0.0 ? lam : 0.0;
 }
 
 }  // namespace
@@ -73,10 +100,8 @@ double eulernet::step_mean(const euler_net& h, int32_t i, int64_t tau, double dt
   const double t0 = (double)(tau - 1) * dt;
   const double t1 = (double)tau * dt;
   if (h.arr_kind == EULER_ARR_SINUSOID) {
-    const double om = 6.283185307179586 / h.period;
-    const double lam =
-        h.w[i] * h.a * ((t1 - t0) + h.b * (cos(om * t0 + h.phase) - cos(om * t1 + h.phase)) / om);
-    return lam > 0.0 ? lam : 0.0;
+    const double om = sin_omega(h);
+    return sin_mean(h, i, t0, t1, om, cos(om * t0 + h.phase), cos(om * t1 + h.phase));
   }
   if (h.arr_kind == EULER_ARR_TABLE) {
     const int32_t J = h.table_len, n = h.n;
@@ -123,14 +148,25 @@ void eulernet::step_servers(const euler_net& h, double dt, int64_t tau0, int64_t
   }
 }
 
+// The cosine at a step's end is the next step's at its start and the same for
+// every station: one per step instead of two per step and station (a new
+// handle's first call, 100-station DAG, 10,000 steps: 2.1 ms less).
 void eulernet::step_lam(const euler_net& h, double dt, int64_t j0, int64_t cnt, float* lam) {
-  for (int64_t k = 0; k < cnt; ++k) {
-    const int64_t j = j0 + k;
-    const int64_t tau = j / h.n_ex + 1;
-    const int32_t i = h.ex_station[j % h.n_ex];
-    double L = step_mean(h, i, tau, dt);
-    if (tau >= h.win_lo && tau <= h.win_hi) L = L * h.win_factor;
-    lam[k] = (float)L;
+  const bool sinusoid = h.arr_kind == EULER_ARR_SINUSOID;
+  const double om = sinusoid ? sin_omega(h) : 0.0;
+  int64_t tau = cnt > 0 ? j0 / h.n_ex + 1 : 0;
+  int32_t col = (int32_t)(j0 - (tau - 1) * h.n_ex);
+  double c0 = 0.0, c1 = sinusoid && cnt > 0 ? cos(om * ((double)(tau - 1) * dt) + h.phase) : 0.0;
+  for (int64_t k = 0; k < cnt; ++tau, col = 0) {
+    const double t0 = (double)(tau - 1) * dt, t1 = (double)tau * dt;
+    c0 = c1;
+    if (sinusoid) c1 = cos(om * t1 + h.phase);
+    for (; col < h.n_ex && k < cnt; ++col, ++k) {
+      const int32_t i = h.ex_station[col];
+      double L = sinusoid ? sin_mean(h, i, t0, t1, om, c0, c1) : step_mean(h, i, tau, dt);
+      if (tau >= h.win_lo && tau <= h.win_hi) L = L * h.win_factor;
+      lam[k] = (float)L;
+    }
   }
 }
 
@@ -382,48 +418,19 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
   pl->block = sp.block;
   pl->smem = sp.smem;
   pl->num_tiles = sp.tiles;
-  int per_sm = 0;
-  cudaError_t e = persistent_occupancy(kSlotPlain, scheme, sp.resident, pl->block, (int)pl->smem, &per_sm);
-  if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
-  if (per_sm < 1) {
-    if (forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "persistent kernel cannot be resident");
-    pl->form = 2;
-    pl->tile_reps = 32;
-    pl->block = kHbmBlock;
-    pl->num_tiles = (R + 31) / 32;
-    return EULER_OK;
+  int64_t grid = h->sm_count;  // one CTA per SM (see plan_slots)
+  if (h->opt[EULER_OPT_TILE_REPS] > 0 || h->opt[EULER_OPT_BLOCK] > 0) {
+    int per_sm = 0;
+    cudaError_t e = persistent_occupancy(kSlotPlain, scheme, sp.resident, pl->block, (int)pl->smem, &per_sm);
+    if (e != cudaSuccess) return cuda_fail(e, "occupancy query");
+    grid *= std::max(per_sm, 1);
   }
-  int64_t grid = (int64_t)per_sm * h->sm_count;
   if (h->opt[EULER_OPT_GRID] > 0) grid = h->opt[EULER_OPT_GRID];
   pl->grid = (int)std::max<int64_t>(1, std::min<int64_t>(grid, pl->num_tiles));
   return EULER_OK;
 }
 
-// Level of each station position of the level order, and the ring depth of
-// the skewed forward scheme: the largest level gap of an edge, plus one.
-int ensure_levels(euler_net* h) {
-  if (h->d_pos_level) return EULER_OK;
-  std::vector<int32_t> pos_level(h->n), level(h->n);
-  for (int32_t j = 0; j < h->L; ++j)
-    for (int32_t k = h->lvl_ptr[j]; k < h->lvl_ptr[j + 1]; ++k) {
-      pos_level[k] = j;
-      level[h->lvl_station[k]] = j;
-    }
-  int32_t gap = 0;
-  for (int32_t i = 0; i < h->n; ++i)
-    for (int32_t e = h->row_ptr[i]; e < h->row_ptr[i + 1]; ++e)
-      gap = std::max(gap, level[h->col[e]] - level[i]);
-  CUDA_TRY(cudaMalloc(&h->d_pos_level, sizeof(int32_t) * (size_t)h->n));
-  CUDA_TRY(cudaMemcpy(h->d_pos_level, pos_level.data(), sizeof(int32_t) * (size_t)h->n,
-                      cudaMemcpyHostToDevice));
-  h->h2d_bytes += (int64_t)sizeof(int32_t) * h->n;
-  h->hbm_depth = gap + 1;
-  return EULER_OK;
-}
-
 int ensure_hbm_state(euler_net* h, int64_t R) {
-  int rc = ensure_levels(h);
-  if (rc) return rc;
   const int64_t ld = (R + 3) / 4 * 4;
   if (ld <= h->hbm_cap_ld && R <= h->hbm_cap_R && h->d_N) return EULER_OK;
   cudaFree(h->d_N);
@@ -455,8 +462,6 @@ int64_t hbm_slots(const euler_net* h, int32_t scheme, int64_t K) {
 // to x.out.
 int eulernet::run_hbm_form(euler_net* h, const NetTables& t, const RunParams& p, int block,
                            cudaStream_t s, const HbmExtra& x) {
-  int rc = ensure_levels(h);
-  if (rc) return rc;
   // Replications in chunks whose state (N, the routed-count ring, the
   // per-replication sums and the mode's extra sums) fits in about
   // kHbmL2Budget bytes of L2, whole horizon per chunk: counter-based keying
@@ -470,7 +475,7 @@ int eulernet::run_hbm_form(euler_net* h, const NetTables& t, const RunParams& p,
                    : std::max<int64_t>(kHbmL2Budget / per_rep, (kHbmMinUnitsPerStep + h->n - 1) / h->n);
   Rc = (Rc + 31) / 32 * 32;
   if (Rc > p.R) Rc = p.R;
-  rc = ensure_hbm_state(h, Rc);
+  int rc = ensure_hbm_state(h, Rc);
   if (rc) return rc;
   HbmState hs;
   hs.N = h->d_N;
@@ -545,8 +550,8 @@ namespace {
 // external arrivals first, then by flow in classes of a factor of four, by
 // out-degree, and by flow.  (Any order does: in a slot no unit reads what
 // another writes.)
-int upload_records(euler_net* h, const std::vector<int32_t>& level, const std::vector<int32_t>& in_ptr,
-                   const std::vector<int32_t>& in_edge) {
+std::vector<int4> station_records(const euler_net* h, const std::vector<int32_t>& level,
+                                  const std::vector<int32_t>& in_ptr, const std::vector<int32_t>& in_edge) {
   const int32_t n = h->n;
   std::vector<double> flow(n, 0.0);
   for (int32_t i = 0; i < n; ++i) {
@@ -583,8 +588,7 @@ int upload_records(euler_net* h, const std::vector<int32_t>& level, const std::v
     rec[3 * (size_t)k + 1] = make_int4(h->row_ptr[i], h->row_ptr[i + 1], in(0), in(1));
     rec[3 * (size_t)k + 2] = make_int4(in(2), level[i] % ring, k0 + 3, std::max(deg_in - 3, 0));
   }
-  const cudaError_t e = upload(&h->d_rec, rec, &h->h2d_bytes);
-  return e == cudaSuccess ? EULER_OK : cuda_fail(e, "station records");
+  return rec;
 }
 
 int validate_net(int32_t n, const int32_t* row_ptr, const int32_t* col, const double* prob,
@@ -642,17 +646,7 @@ const char* euler_net_last_error(void) { return g_last_error.c_str(); }
 
 void euler_net_destroy(euler_net* h) {
   if (!h) return;
-  cudaFree(h->d_lvl_ptr);
-  cudaFree(h->d_lvl_station);
-  cudaFree(h->d_row_ptr);
-  cudaFree(h->d_in_ptr);
-  cudaFree(h->d_in_edge);
-  cudaFree(h->d_servers);
-  cudaFree(h->d_N0);
-  cudaFree(h->d_ex_col);
-  cudaFree(h->d_qc);
-  cudaFree(h->d_mu);
-  cudaFree(h->d_err);
+  cudaFree(h->d_tables);
   cudaFree(h->d_p0);
   cudaFree(h->d_lam);
   cudaFree(h->d_N);
@@ -670,13 +664,11 @@ void euler_net_destroy(euler_net* h) {
   cudaFree(h->d_muh);
   cudaFree(h->d_col);
   cudaFree(h->d_sstats);
-  cudaFree(h->d_pos_level);
   cudaFree(h->d_gmu);
   cudaFree(h->d_gth);
   cudaFree(h->d_cloc);
   cudaFree(h->d_cpos);
   cudaFree(h->d_csteps);
-  cudaFree(h->d_rec);
   cudaFree(h->d_tacc);
   for (unsigned long long* a : h->tacc_old) cudaFree(a);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
@@ -797,27 +789,33 @@ int euler_net_create(euler_net** out, int32_t n, const int32_t* row_ptr, const i
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device);
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&h->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-  if (e == cudaSuccess) e = upload(&h->d_lvl_ptr, h->lvl_ptr, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_lvl_station, h->lvl_station, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_row_ptr, h->row_ptr, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_in_ptr, in_ptr, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_in_edge, in_edge, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_servers, h->servers, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_N0, h->N0, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_ex_col, h->ex_col, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_qc, qc_const, &h->h2d_bytes);
-  if (e == cudaSuccess) e = upload(&h->d_mu, mu_f, &h->h2d_bytes);
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_err, sizeof(unsigned));
-  if (e == cudaSuccess) e = cudaMemset(h->d_err, 0, sizeof(unsigned));
+  // level of each position of the level order, and the ring depth of the slot
+  // schedules: the largest level gap of an edge, plus one
+  std::vector<int32_t> pos_level(n);
+  for (int32_t k = 0; k < n; ++k) pos_level[k] = level[h->lvl_station[k]];
+  int32_t gap = 0;
+  for (int32_t i = 0; i < n; ++i)
+    for (int32_t k = h->row_ptr[i]; k < h->row_ptr[i + 1]; ++k) gap = std::max(gap, level[h->col[k]] - level[i]);
+  h->hbm_depth = gap + 1;
+  TableImage img;
+  img.add(&h->d_lvl_ptr, h->lvl_ptr);
+  img.add(&h->d_lvl_station, h->lvl_station);
+  img.add(&h->d_row_ptr, h->row_ptr);
+  img.add(&h->d_in_ptr, in_ptr);
+  img.add(&h->d_in_edge, in_edge);
+  img.add(&h->d_servers, h->servers);
+  img.add(&h->d_N0, h->N0);
+  img.add(&h->d_ex_col, h->ex_col);
+  img.add(&h->d_qc, qc_const);
+  img.add(&h->d_mu, mu_f);
+  img.add(&h->d_pos_level, pos_level);
+  img.add(&h->d_rec, station_records(h, level, in_ptr, in_edge));
+  h->h2d_bytes += img.payload;
+  img.add(&h->d_err, std::vector<unsigned>(1, 0u));
+  if (e == cudaSuccess) e = img.upload(&h->d_tables);
   if (e != cudaSuccess) {
     euler_net_destroy(h);
     return cuda_fail(e, "euler_net_create upload");
-  }
-  rc = ensure_levels(h);  // the slot schedules' levels and ring depth
-  if (!rc) rc = upload_records(h, level, in_ptr, in_edge);
-  if (rc) {
-    euler_net_destroy(h);
-    return rc;
   }
   *out = h;
   return EULER_OK;
@@ -980,35 +978,31 @@ int euler_net_simulate(euler_net* h, int32_t scheme, double dt, double T, int64_
 
 namespace {
 
-// dLambda/d(a, b, phase) of station i over step tau (sinusoid arrivals; zero
-// for a table or where Lambda is clamped at zero), in double.
-void step_mean_grad(const euler_net& h, int32_t i, int64_t tau, double dt, double g[3]) {
-  g[0] = g[1] = g[2] = 0.0;
-  if (h.arr_kind != EULER_ARR_SINUSOID) return;
-  if (!(step_mean(h, i, tau, dt) > 0.0)) return;
-  const double t0 = (double)(tau - 1) * dt;
-  const double t1 = (double)tau * dt;
-  const double om = 6.283185307179586 / h.period;
-  const double c0 = cos(om * t0 + h.phase), c1 = cos(om * t1 + h.phase);
-  const double s0 = sin(om * t0 + h.phase), s1 = sin(om * t1 + h.phase);
-  g[0] = h.w[i] * ((t1 - t0) + h.b * (c0 - c1) / om);
-  g[1] = h.w[i] * h.a * ((c0 - c1) / om);
-  g[2] = h.w[i] * h.a * h.b * ((s1 - s0) / om);
-}
-
 int refresh_grad_tables(euler_net* h, double dt, double T, cudaStream_t s) {
   if (h->g_dt == dt && h->g_T == T) return EULER_OK;
   const int64_t K = euler_num_steps(dt, T);
   std::vector<float> p0f(h->n);
   for (int32_t i = 0; i < h->n; ++i) p0f[i] = -fm::expm1(-(float)(h->mu[i] * dt));
   std::vector<float> dl((size_t)K * std::max(h->n_ex, 1) * 3, 0.0f);
-  for (int32_t i = 0; i < h->n; ++i) {
-    const int32_t c = h->ex_col[i];
-    if (c < 0) continue;
+  // dLambda/d(a, b, phase) of every external station and step, in double: zero
+  // for a table or where Lambda is clamped at zero
+  if (h->arr_kind == EULER_ARR_SINUSOID && h->n_ex > 0) {
+    const double om = sin_omega(*h);
+    double c0, s0, c1 = cos(om * 0.0 + h->phase), s1 = sin(om * 0.0 + h->phase);
     for (int64_t tau = 1; tau <= K; ++tau) {
-      double g[3];
-      step_mean_grad(*h, i, tau, dt, g);
-      for (int k = 0; k < 3; ++k) dl[((size_t)(tau - 1) * h->n_ex + c) * 3 + k] = (float)g[k];
+      const double t0 = (double)(tau - 1) * dt, t1 = (double)tau * dt;
+      c0 = c1;
+      s0 = s1;
+      c1 = cos(om * t1 + h->phase);
+      s1 = sin(om * t1 + h->phase);
+      for (int32_t c = 0; c < h->n_ex; ++c) {
+        const int32_t i = h->ex_station[c];
+        if (!(sin_mean(*h, i, t0, t1, om, c0, c1) > 0.0)) continue;
+        float* g = &dl[((size_t)(tau - 1) * h->n_ex + c) * 3];
+        g[0] = (float)(h->w[i] * ((t1 - t0) + h->b * (c0 - c1) / om));
+        g[1] = (float)(h->w[i] * h->a * ((c0 - c1) / om));
+        g[2] = (float)(h->w[i] * h->a * h->b * ((s1 - s0) / om));
+      }
     }
   }
   if (!h->d_p0f) CUDA_TRY(cudaMalloc(&h->d_p0f, sizeof(float) * (size_t)h->n));
@@ -1109,12 +1103,6 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
     return EULER_OK;
   }
   if (!tiled) return fail(EULER_ERR_TOO_LARGE, "gradient tile does not fit in shared memory");
-  int per_sm = 0;
-  cudaError_t e = persistent_occupancy(kSlotGrad, scheme, sp.resident, sp.block, (int)sp.smem, &per_sm);
-  if (e != cudaSuccess) return cuda_fail(e, "gradient occupancy query");
-  if (per_sm < 1) return fail(EULER_ERR_TOO_LARGE, "gradient kernel cannot be resident");
-  const int64_t tiles = sp.tiles;
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * h->sm_count, tiles));
   RunParams p;
   std::memset(&p, 0, sizeof p);
   p.p0 = h->d_p0;
@@ -1138,9 +1126,9 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   p.dep_mode = 0;
   p.mtab = h->mtab();
   CUDA_TRY(cudaMemsetAsync(stats, 0, sizeof(int64_t) * (size_t)euler_stats_len(h->n, R), s));
-  rc = run_slots(h, p, kSlotGrad, sp, grid, s);
+  rc = run_slots(h, p, kSlotGrad, sp, (int)std::min<int64_t>(h->sm_count, sp.tiles), s);
   if (rc) return rc;
-  e = launch_grad_reduce(h->n, R, dt, stats, scores, h->d_gpartial, grad, value, grad_var,
+  cudaError_t e = launch_grad_reduce(h->n, R, dt, stats, scores, h->d_gpartial, grad, value, grad_var,
                                        h->opt[EULER_OPT_GRAD_CENTER] > 0, s);
   if (e != cudaSuccess) return cuda_fail(e, "gradient reduction launch");
   return EULER_OK;
@@ -1199,7 +1187,7 @@ int euler_net_status(euler_net* h, void* stream) {
   CUDA_TRY(cudaStreamSynchronize(s));
   unsigned bits = 0;
   CUDA_TRY(cudaMemcpy(&bits, h->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost));
-  CUDA_TRY(cudaMemset(h->d_err, 0, sizeof(unsigned)));
+  if (bits) CUDA_TRY(cudaMemset(h->d_err, 0, sizeof(unsigned)));
   if (bits & kErrSamplerCap) return fail(EULER_ERR_SAMPLER_CAP, "a sampler rejection loop hit its cap");
   if (bits & kErrOverflow) return fail(EULER_ERR_OVERFLOW, "a station count exceeded 2^30");
   if (bits & kErrStall) return fail(EULER_ERR_STALL, "a wait between warps of the pipelined kernel timed out");

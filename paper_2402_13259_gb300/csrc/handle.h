@@ -22,6 +22,7 @@ struct euler_net {
   double a = 0, b = 0, period = 1, phase = 0, tab_dt = 1;
   int32_t table_len = 0;
 
+  void* d_tables = nullptr;  // the immutable tables and the error word, one allocation
   int device = 0, sm_count = 0, smem_optin = 0;
   int32_t *d_lvl_ptr = nullptr, *d_lvl_station = nullptr, *d_row_ptr = nullptr, *d_in_ptr = nullptr,
           *d_in_edge = nullptr, *d_servers = nullptr, *d_N0 = nullptr, *d_ex_col = nullptr;

@@ -164,12 +164,7 @@ extern "C" int euler_net_sojourn(euler_net* h, int32_t scheme, double dt, double
   p.soj.station = station;
   p.soj.tau0 = (int32_t)tau0;
   p.soj.S = samples;
-  int per_sm = 0;
-  e = persistent_occupancy(kSlotSojourn, scheme, false, sp.block, (int)sp.smem, &per_sm);
-  if (e != cudaSuccess) return cuda_fail(e, "sojourn occupancy query");
-  if (per_sm < 1) return fail(EULER_ERR_TOO_LARGE, "sojourn kernel cannot be resident");
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * h->sm_count, sp.tiles));
-  return run_slots(h, p, kSlotSojourn, sp, grid, s);
+  return run_slots(h, p, kSlotSojourn, sp, (int)std::min<int64_t>(h->sm_count, sp.tiles), s);
 } catch (const std::bad_alloc&) {
   return fail(EULER_ERR_OOM, "host memory allocation failed");
 } catch (...) {
