@@ -298,8 +298,8 @@ typedef struct euler_batch euler_batch; /* opaque */
  * alive until euler_batch_destroy).  A handle may appear several times only
  * with the same (dt, T).  A network with n x replications >= 2^18 units per
  * step (the threshold the autotuner may move) fills the GPU by itself and
- * runs in the HBM form of euler_net_simulate (per-step kernels replayed from
- * CUDA graphs), these networks one after another; the others share one
+ * runs as a euler_net_simulate call does (in the persistent or the HBM form),
+ * these networks one after another; the others share one
  * persistent launch whose work items are (network, tile of replications),
  * ordered by decreasing cost, with per-network tile sizes that fill the
  * block.  Errors: EULER_ERR_ARG, EULER_ERR_TOO_LARGE (a network whose

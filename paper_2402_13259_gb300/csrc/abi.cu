@@ -173,8 +173,7 @@ void eulernet::step_lam(const euler_net& h, double dt, int64_t j0, int64_t cnt, 
 // The persistent form's per-unit sums for `grid` CTAs, into p.  Grown by
 // doubling and kept until the handle goes: a graph captured from an earlier
 // call may hold the former array, and a call may itself be under capture.
-static int slot_scratch(euler_net* h, int grid, int Rt, RunParams* p) {
-  p->acc_stride = slot_acc_len(h->n, h->n_ex, Rt);
+static int slot_scratch(euler_net* h, int grid, RunParams* p) {
   const size_t need = (size_t)(p->acc_stride * grid);
   if (need > h->tacc_cap) {
     const size_t len = std::max(need, 2 * h->tacc_cap);
@@ -193,14 +192,18 @@ static int slot_scratch(euler_net* h, int grid, int Rt, RunParams* p) {
 }
 
 // The launches of a persistent-form run (see SlotPlan): p complete but for what
-// the plan decides.  One launch covers at most about 2e10 station-step updates
+// the plan decides (p.acc: the caller's per-unit sums, or nullptr for the
+// handle's).  One launch covers at most about 2e10 station-step updates
 // (about a second), a whole number of waves of tiles.
 int eulernet::run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp, int grid, cudaStream_t s) {
   p.tile_reps = sp.Rt;
   p.task_lanes = sp.lanes;
   p.task_inline = sp.in_place;
-  const int rc = slot_scratch(h, grid, sp.Rt, &p);
-  if (rc) return rc;
+  p.acc_stride = slot_acc_len(h->n, h->n_ex, sp.Rt);
+  if (!p.acc) {
+    const int rc = slot_scratch(h, grid, &p);
+    if (rc) return rc;
+  }
   const double wave = (double)h->n * (double)sp.Rt * (double)p.K * grid;
   const int64_t step = (int64_t)grid * std::max<int64_t>(1, (int64_t)(2e10 / wave));
   for (int64_t t0 = 0; t0 < sp.tiles; t0 += step) {
@@ -325,6 +328,10 @@ bool eulernet::plan_slots(const euler_net* h, int64_t R, bool grad, int32_t soj,
 // s = 10 .. 10,000) to 1.6 times (100 stations) as fast.
 bool eulernet::hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp) {
   return (int64_t)h->n * R >= kHbmMinUnitsPerStep && sp.fill < kTileMinFill;
+}
+
+bool eulernet::plan_alone(const euler_net* h, int64_t R, SlotPlan* sp) {
+  return plan_slots(h, R, false, 0, 0, 0, sp) && !hbm_beats_tiles(h, R, *sp);
 }
 
 namespace {
@@ -923,15 +930,20 @@ RunParams simulate_params(const euler_net* h, int32_t scheme, double dt, int64_t
 
 }  // namespace
 
-int eulernet::simulate_hbm(euler_net* h, int32_t scheme, double dt, double T, int64_t R, uint64_t seed,
-                           int64_t rep_begin, int64_t* stats, cudaStream_t s, int block, int graph_steps,
-                           int64_t k_limit) {
+int eulernet::simulate_alone(euler_net* h, int32_t scheme, double dt, double T, int64_t R, uint64_t seed,
+                             int64_t rep_begin, int64_t* stats, cudaStream_t s, int block, int graph_steps,
+                             int64_t k_limit, unsigned long long* acc) {
   int rc = refresh_step_tables(h, dt, T, s);
   if (rc) return rc;
   int64_t K = euler_num_steps(dt, T);
   if (k_limit > 0 && K > k_limit) K = k_limit;
   if (R == 0) return EULER_OK;
-  const RunParams p = simulate_params(h, scheme, dt, K, R, seed, rep_begin, stats, 32, (R + 31) / 32);
+  RunParams p = simulate_params(h, scheme, dt, K, R, seed, rep_begin, stats, 32, (R + 31) / 32);
+  SlotPlan sp;
+  if (acc && plan_alone(h, R, &sp)) {
+    p.acc = acc;
+    return run_slots(h, p, kSlotPlain, sp, (int)std::min<int64_t>(h->sm_count, sp.tiles), s);
+  }
   HbmExtra x;
   x.graph_steps = graph_steps;
   return run_hbm_form(h, h->tables(), p, block, s, x);

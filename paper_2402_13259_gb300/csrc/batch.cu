@@ -3,10 +3,10 @@
 // replayed from a CUDA graph.
 //
 // Two kinds of networks.  A network with n_j R_j >= hbm_min_units units per
-// step fills the GPU by itself: it runs in the HBM form, the per-step kernels
-// of euler_net_simulate (one warp per station and 32 replications, a CUDA
-// graph of slots replayed to its horizon), one such network after another.
-// The others share one persistent launch fed by a work queue.
+// step fills the GPU by itself: it runs as a euler_net_simulate call does, in
+// the persistent or the HBM form, one such network after another (64 mixed
+// networks 67.6 ms; with these in the HBM form 74.3 ms).  The others share one
+// persistent launch fed by a work queue.
 //
 // Work item = (network j, tile of replications).  Network j gets a tile size
 // Rt_j (a power of two) so that its widest phase keeps the block busy
@@ -39,7 +39,7 @@ struct euler_batch {
   std::vector<euler_net*> nets;
   std::vector<euler_run> runs;
   int device = 0, sm_count = 0, smem_optin = 0;
-  // networks run in the HBM form, and its launch shape
+  // networks run by themselves, and the HBM form's launch shape for those that take it
   std::vector<int> hbm_nets;
   std::vector<char> is_hbm;  // per network
   int64_t hbm_min_units = kHbmMinUnitsPerStep;
@@ -65,6 +65,8 @@ struct euler_batch {
   int* d_counter = nullptr;
   unsigned long long* d_sacc = nullptr;  // the CTAs' per-unit sums
   size_t sacc_cap = 0;
+  unsigned long long* d_alone = nullptr;  // the per-unit sums of the networks run by themselves, one after another
+  size_t alone_cap = 0;
   // graph of the last run
   cudaGraphExec_t exec = nullptr;
   std::vector<int64_t*> graph_stats;
@@ -130,7 +132,7 @@ bool tile_for(const euler_batch* b, int j, int block, int64_t cap, int rt_shift,
 // network's whole horizon on one CTA, so when the launch has more items than
 // CTAs, a network whose item costs (n K Rt) more than cp_factor x the mean
 // load per CTA (sum of n K R over the launch's networks / CTAs) would outlast
-// the rest of the launch; such a network runs in the HBM form instead, where
+// the rest of the launch; such a network runs by itself instead, where
 // one step of all its replications spreads over the whole GPU, provided a
 // step has at least 2^14 units (512 warps) so that its launches do more than
 // wait on launch latency.  With fewer items than CTAs every item runs at
@@ -153,7 +155,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
     const euler_net* h = b->nets[j];
     if (288 + 4 * ((int64_t)h->n + (int64_t)h->tables().ring * h->E) > cap)
       return bfail(EULER_ERR_TOO_LARGE, "a network's state of one replication does not fit the shared-memory budget");
-    // a tile whose lists and arrivals do not fit beside the state: HBM form
+    // a tile whose lists and arrivals do not fit beside the state: by itself
     if (!tile_for(b, j, block, cap, rt_shift, &Rt_of[j])) b->is_hbm[j] = 1;
   }
   if (cp_factor > 0.0) {
@@ -263,6 +265,19 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
     BTRY(cudaMalloc(&b->d_sacc, sizeof(unsigned long long) * sacc_need));
     b->sacc_cap = sacc_need;
   }
+  size_t alone_need = 0;
+  for (int j : b->hbm_nets) {
+    const euler_net* h = b->nets[j];
+    SlotPlan sp;
+    if (plan_alone(h, b->runs[j].replications, &sp))
+      alone_need = std::max(alone_need, (size_t)(slot_acc_len(h->n, h->n_ex, sp.Rt) * std::min<int64_t>(h->sm_count, sp.tiles)));
+  }
+  if (alone_need > b->alone_cap) {
+    cudaFree(b->d_alone);
+    b->d_alone = nullptr;
+    BTRY(cudaMalloc(&b->d_alone, sizeof(unsigned long long) * alone_need));
+    b->alone_cap = alone_need;
+  }
   BTRY(cudaMemcpy(b->d_nets, b->h_nets.data(), sizeof(NetTables) * b->count, cudaMemcpyHostToDevice));
   if (b->num_items)
     BTRY(cudaMemcpy(b->d_items, b->h_items.data(), sizeof(int2) * b->num_items, cudaMemcpyHostToDevice));
@@ -294,15 +309,16 @@ int upload_runs(euler_batch* b, int64_t* const* stats, double k_scale) {
   return EULER_OK;
 }
 
-// The networks of the HBM form, one after another on stream s (horizons
+// The networks run by themselves, one after another on stream s (horizons
 // scaled by k_scale for tuning; only the networks in `subset` when it is not
 // null).
 int run_hbm_nets(euler_batch* b, int64_t* const* stats, cudaStream_t s, double k_scale,
                  const std::vector<int>* subset = nullptr) {
   for (int j : subset ? *subset : b->hbm_nets) {
     const euler_run& r = b->runs[j];
-    const int rc = simulate_hbm(b->nets[j], r.scheme, r.dt, r.T, r.replications, r.seed, r.rep_begin, stats[j], s,
-                                b->hbm_block, b->hbm_graph_steps, k_scale > 0.0 ? scaled_steps(b, j, k_scale) : 0);
+    const int rc = simulate_alone(b->nets[j], r.scheme, r.dt, r.T, r.replications, r.seed, r.rep_begin, stats[j], s,
+                                  b->hbm_block, b->hbm_graph_steps, k_scale > 0.0 ? scaled_steps(b, j, k_scale) : 0,
+                                  b->d_alone);
     if (rc) return rc;
   }
   return EULER_OK;
@@ -618,6 +634,7 @@ void euler_batch_destroy(euler_batch* b) {
   cudaFree(b->d_items);
   cudaFree(b->d_counter);
   cudaFree(b->d_sacc);
+  cudaFree(b->d_alone);
   delete b;
 }
 

@@ -171,14 +171,19 @@ bool plan_slots(const euler_net* h, int64_t R, bool grad, int32_t soj, int force
 bool hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp);
 int run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp, int grid, cudaStream_t s);
 
-// A plain simulation call in the HBM form (the per-step kernels; the batched
-// form's large networks): tables made current for (dt, T), `block` threads
-// per step kernel, `graph_steps` slots per graph replay (0: default), at most
-// k_limit steps when k_limit > 0 (tuning runs).  `stats` must be zeroed by
-// the caller, on stream s.
-int simulate_hbm(euler_net* h, int32_t scheme, double dt, double T, int64_t R, uint64_t seed,
-                 int64_t rep_begin, int64_t* stats, cudaStream_t s, int block, int graph_steps,
-                 int64_t k_limit);
+// Whether a plain run of R replications takes the persistent form, with *sp
+// its plan, or the HBM form.
+bool plan_alone(const euler_net* h, int64_t R, SlotPlan* sp);
+
+// A plain simulation call of a network that fills the GPU by itself (the
+// batched form's large networks), in the form of plan_alone: tables made
+// current for (dt, T); `acc` the persistent form's per-unit sums (HBM form if
+// nullptr); `block` threads per step kernel and `graph_steps` slots per graph
+// replay (0: default) of the HBM form; at most k_limit steps when k_limit > 0
+// (tuning runs).  `stats` must be zeroed by the caller, on stream s.
+int simulate_alone(euler_net* h, int32_t scheme, double dt, double T, int64_t R, uint64_t seed,
+                   int64_t rep_begin, int64_t* stats, cudaStream_t s, int block, int graph_steps,
+                   int64_t k_limit, unsigned long long* acc);
 
 // Per-step mean of the external arrivals of station i over step tau: the
 // exact integral of lambda_i over ((tau-1) dt, tau dt] (Sec. 2.1.1), in double.
