@@ -36,12 +36,10 @@ sys.path.insert(0, ROOT)
 METRIC = "station-step updates/s per GB300 (fwd/bwd Euler), % of binding roofline"
 UNIT = "station-step updates/s"
 LANES_PER_SM = 128  # instruction issue: 4 schedulers x 32 lanes per clock
-# DRAM bytes of one simulate call (mean of the two schemes) from one ncu
-# capture of the step kernels: 11.917 MB (fused backward) and 11.938 MB
-# (skewed forward) per step launch at steady state, x 10,001 and 10,009 step
-# launches per call.  Valid only for the kernel sources with this hash and
-# the launch forms listed; reported as null otherwise.
-TRAFFIC = {"hash": "25feb6e182f56b21", "forms": [2, 2], "bytes_per_call": 0.5 * (11.917e6 * 10001 + 11.938e6 * 10009)}
+# DRAM bytes of one simulate call (mean of the two schemes) from an ncu
+# capture, valid only for the kernel sources with this hash and the launch
+# forms listed; none is held for the present sources, so null is reported.
+TRAFFIC = {"hash": None, "forms": [1, 1], "bytes_per_call": None}
 
 
 def sm_count(device: int = 0) -> int:
@@ -76,7 +74,7 @@ def host_cpu() -> dict:
 
 def kernel_hash() -> str:
     h = hashlib.sha256()
-    for f in ("hbm_step.cuh", "unit.cuh", "sampling.cuh"):
+    for f in ("tile_slots.cuh", "hbm_step.cuh", "unit.cuh", "sampling.cuh"):
         with open(os.path.join(ROOT, "paper_2402_13259_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -777,7 +775,8 @@ def main():
                 "traffic": TRAFFIC["bytes_per_call"] if valid else None,
                 "kernel": "hbm_phase_kernel (per-step kernels of one simulate call, CUDA graph)" if hbm
                           else "persistent_kernel",
-                "launch": "one euler_net_simulate call per scheme (kernel time + graph launch gaps)",
+                "launch": "one euler_net_simulate call per scheme (kernel time" +
+                          (" + graph launch gaps)" if hbm else ")"),
                 "ops_per_unit": {k: v["ops_per_unit"] for k, v in per_scheme.items()},
                 "peak_note": f"{sms} SMs (device attribute) x {LANES_PER_SM} lanes x {sm_max:.0f} MHz "
                              "(nvidia-smi max SM clock; issue rate)"}
