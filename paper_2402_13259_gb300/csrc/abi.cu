@@ -805,7 +805,6 @@ int euler_net_create(euler_net** out, int32_t n, const int32_t* row_ptr, const i
     for (int32_t k = h->row_ptr[i]; k < h->row_ptr[i + 1]; ++k) gap = std::max(gap, level[h->col[k]] - level[i]);
   h->hbm_depth = gap + 1;
   TableImage img;
-  img.add(&h->d_lvl_ptr, h->lvl_ptr);
   img.add(&h->d_lvl_station, h->lvl_station);
   img.add(&h->d_row_ptr, h->row_ptr);
   img.add(&h->d_in_ptr, in_ptr);

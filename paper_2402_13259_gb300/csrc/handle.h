@@ -24,7 +24,7 @@ struct euler_net {
 
   void* d_tables = nullptr;  // the immutable tables and the error word, one allocation
   int device = 0, sm_count = 0, smem_optin = 0;
-  int32_t *d_lvl_ptr = nullptr, *d_lvl_station = nullptr, *d_row_ptr = nullptr, *d_in_ptr = nullptr,
+  int32_t *d_lvl_station = nullptr, *d_row_ptr = nullptr, *d_in_ptr = nullptr,
           *d_in_edge = nullptr, *d_servers = nullptr, *d_N0 = nullptr, *d_ex_col = nullptr;
   float4* d_qc = nullptr;
   float* d_mu = nullptr;
@@ -109,8 +109,6 @@ struct euler_net {
     t.n = n;
     t.E = E;
     t.L = L;
-    t.max_level = max_level;
-    t.lvl_ptr = d_lvl_ptr;
     t.lvl_station = d_lvl_station;
     t.row_ptr = d_row_ptr;
     t.qc = d_qc;

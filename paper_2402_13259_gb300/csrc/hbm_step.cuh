@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256, EN_HBM_MIN_BLOCKS) hbm_phase_kernel(NetTa
         v[0] = o.D; v[1] = o.X; v[2] = o.A;
         part[1] += o.D; part[2] += o.X; part[3] += o.A;
       }
-      reduce_to<3>(st + 2, v, lead, 32, true);
+      reduce_to<3>(st + 2, v, lead, true);
     } else if constexpr (phase == 1) {  // backward gather / update
       int32_t v[2] = {0, 0};
       if (act) {
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(256, EN_HBM_MIN_BLOCKS) hbm_phase_kernel(NetTa
         v[0] = nn; v[1] = nn < c ? nn : c;
         part[0] += nn;
       }
-      reduce_to<2>(st, v, lead, 32, true);
+      reduce_to<2>(st, v, lead, true);
     } else if constexpr (phase == 4) {  // backward, fused: gather tau - 1, then draw tau
       int32_t v[5] = {0, 0, 0, 0, 0};
       if (act) {
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(256, EN_HBM_MIN_BLOCKS) hbm_phase_kernel(NetTa
           }
         }
       }
-      reduce_to<5>(st, v, lead, 32, true);
+      reduce_to<5>(st, v, lead, true);
     } else {  // forward: one level (2) or a skewed slot (3)
       int32_t v[5] = {0, 0, 0, 0, 0};
       if (act) {
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(256, EN_HBM_MIN_BLOCKS) hbm_phase_kernel(NetTa
         v[0] = o.N; v[1] = o.N < c ? o.N : c; v[2] = o.D; v[3] = o.X; v[4] = o.A;
         part[0] += o.N; part[1] += o.D; part[2] += o.X; part[3] += o.A;
       }
-      reduce_to<5>(st, v, lead, 32, true);
+      reduce_to<5>(st, v, lead, true);
     }
   }
   if (rok) {

@@ -13,8 +13,6 @@ struct NetTables {
   int32_t n;          // stations
   int32_t E;          // edges (CSR nnz)
   int32_t L;          // levels (longest-path depth + 1)
-  int32_t max_level;  // stations in the widest level
-  const int32_t* lvl_ptr;      // [L+1] offsets into lvl_station
   const int32_t* lvl_station;  // [n] stations ordered by (level, index)
   const int32_t* row_ptr;      // [n+1] CSR (routing P)
   const float4* qc;            // [E] BinomConst of each edge's conditional split probability

@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(512, 2) pipeline_kernel(NetTables t, RunParams
             x_r += o.X;
             a_r += o.A;
           }
-          reduce_to<5>(sacc + 6 * (int64_t)i, v, lead, 32, false);
+          reduce_to<5>(sacc + 6 * (int64_t)i, v, lead, false);
         }
         publish(ph1, w, tau, mute);
         publish(done, w, tau, mute);
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(512, 2) pipeline_kernel(NetTables t, RunParams
             x_r += o.X;
             a_r += o.A;
           }
-          reduce_to<3>(sacc + 6 * (int64_t)i + 2, v, lead, 32, false);
+          reduce_to<3>(sacc + 6 * (int64_t)i + 2, v, lead, false);
         }
         publish(ph1, w, tau, mute);
         ok = ok && wait_mask(ph1, prod, tau, lim, zz);
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(512, 2) pipeline_kernel(NetTables t, RunParams
             v[1] = nn < c ? nn : c;
             q_r += nn;
           }
-          reduce_to<2>(sacc + 6 * (int64_t)i, v, lead, 32, false);
+          reduce_to<2>(sacc + 6 * (int64_t)i, v, lead, false);
         }
         publish(done, w, tau, mute);
       }
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(512, 2) pipeline_kernel(NetTables t, RunParams
     for (int k = k_begin; k < k_end; ++k) {
       const int32_t i = __ldg(t.lvl_station + k);
       int32_t v[1] = {rvalid ? Ns[(int64_t)i * kPipeTile + lane] : 0};
-      reduce_to<1>(sacc + 6 * (int64_t)i + 5, v, lead, 32, false);
+      reduce_to<1>(sacc + 6 * (int64_t)i + 5, v, lead, false);
     }
     __syncthreads();
     int64_t* st_rep = p.stats + 5 * (int64_t)n;

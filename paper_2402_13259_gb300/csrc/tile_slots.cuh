@@ -431,7 +431,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
     }
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      const long long v = seg_sum64(s[k], 32);
+      const long long v = warp_sum64(s[k]);
       if (lane == 0 && v)
         atomicAdd(reinterpret_cast<unsigned long long*>(k < 5 ? p.stats + 5 * (int64_t)ra.x + k : st_nk + ra.x),
                   (unsigned long long)v);

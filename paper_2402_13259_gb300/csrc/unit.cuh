@@ -34,26 +34,16 @@ __device__ __forceinline__ int64_t gather_in(const NetTables& t, int32_t i, cons
   return s;
 }
 
-// Sum `v` over aligned segments of `w` lanes (w a power of two <= 32); the
-// segment total ends up in every lane of the segment.
-__device__ __forceinline__ unsigned seg_sum32(unsigned v, int w) {
-  if (w == 32) return __reduce_add_sync(kFull, v);
-  for (int off = w >> 1; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
+// Sum of a warp's 64-bit values, in every lane.
+__device__ __forceinline__ long long warp_sum64(long long v) {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
   return v;
 }
 
-__device__ __forceinline__ long long seg_sum64(long long v, int w) {
-  for (int off = w >> 1; off > 0; off >>= 1) v += __shfl_xor_sync(kFull, v, off);
-  return v;
-}
-
-// Reduce NV per-unit values over the replication segment and add them to
-// dst[0..NV) by the segment leader.  `fits` must be warp-uniform-safe: it is
-// combined with __all_sync here.  mode 0: plain add (exclusive owner), 1:
-// shared/global atomic add.
+// Reduce NV per-unit values over the warp and add them to dst[0..NV) by its
+// lead lane: a plain add (exclusive owner) or an atomic one.
 template <int NV>
-__device__ __forceinline__ void reduce_to(long long* dst, const int32_t (&v)[NV], bool lead,
-                                          int w, bool atomic) {
+__device__ __forceinline__ void reduce_to(long long* dst, const int32_t (&v)[NV], bool lead, bool atomic) {
   int32_t vmax = 0;
 #pragma unroll
   for (int s = 0; s < NV; ++s) vmax = v[s] > vmax ? v[s] : vmax;
@@ -61,10 +51,10 @@ __device__ __forceinline__ void reduce_to(long long* dst, const int32_t (&v)[NV]
   long long tot[NV];
   if (small) {
 #pragma unroll
-    for (int s = 0; s < NV; ++s) tot[s] = (long long)seg_sum32((unsigned)v[s], w);
+    for (int s = 0; s < NV; ++s) tot[s] = (long long)__reduce_add_sync(kFull, (unsigned)v[s]);
   } else {
 #pragma unroll
-    for (int s = 0; s < NV; ++s) tot[s] = seg_sum64((long long)v[s], w);
+    for (int s = 0; s < NV; ++s) tot[s] = warp_sum64((long long)v[s]);
   }
   if (lead) {
 #pragma unroll
