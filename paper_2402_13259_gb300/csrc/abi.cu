@@ -438,7 +438,7 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
 }
 
 int ensure_hbm_state(euler_net* h, int64_t R) {
-  const int64_t ld = (R + 3) / 4 * 4;
+  const int64_t ld = hbm_ld(R);
   if (ld <= h->hbm_cap_ld && R <= h->hbm_cap_R && h->d_N) return EULER_OK;
   cudaFree(h->d_N);
   cudaFree(h->d_Redge);
@@ -489,7 +489,9 @@ int eulernet::run_hbm_form(euler_net* h, const NetTables& t, const RunParams& p,
   hs.Redge = h->d_Redge;
   hs.racc = h->d_racc;
   hs.tau = h->d_tau;
-  hs.ld = h->hbm_cap_ld;
+  // this call's own stride, not that of a larger state kept from an earlier
+  // call: the callers size the extra state by their R, and Rc <= R
+  hs.ld = hbm_ld(Rc);
   hs.pos_level = h->d_pos_level;
   hs.depth = h->hbm_depth;
   hs.mu_acc = x.mu_acc;
@@ -1068,7 +1070,7 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   SlotPlan sp;
   const bool tiled = plan_slots(h, R, true, 0, 0, 0, &sp);
   if (forced == 2 || (forced <= 0 && (tiled ? hbm_beats_tiles(h, R, sp) : (int64_t)h->n * R >= kHbmMinUnitsPerStep))) {
-    const int64_t ld = (R + 3) / 4 * 4;
+    const int64_t ld = hbm_ld(R);
     rc = grow(&h->d_gmu, &h->gmu_cap, (size_t)(h->n * ld));
     if (rc) return rc;
     rc = grow(&h->d_gth, &h->gth_cap, (size_t)(std::max(h->n_ex, 1) * 3 * ld));

@@ -136,6 +136,9 @@ constexpr int kHbmBlock = 256;
 // Bytes of HBM-form state per replication chunk, so that a chunk stays in L2.
 constexpr int64_t kHbmL2Budget = int64_t(64) << 20;
 
+// Leading dimension of the HBM form's state of R replications (16-byte rows).
+inline int64_t hbm_ld(int64_t R) { return (R + 3) / 4 * 4; }
+
 // What an HBM-form run computes besides the statistics (see HbmMode).
 struct HbmExtra {
   int mode = kHbmPlain;

@@ -128,7 +128,7 @@ extern "C" int euler_net_sojourn(euler_net* h, int32_t scheme, double dt, double
   if (forced != 2 && (forced > 0 || !large) && least > h->smem_optin)
     return fail(EULER_ERR_TOO_LARGE, "sojourn tile does not fit in shared memory");
   if (forced == 2 || !tiled || (forced <= 0 && hbm_beats_tiles(h, R, sp))) {
-    const int64_t ld = (R + 3) / 4 * 4;
+    const int64_t ld = hbm_ld(R);
     const size_t need = (size_t)samples * (size_t)ld;
     if (need > h->cust_cap) {
       cudaFree(h->d_cloc);
