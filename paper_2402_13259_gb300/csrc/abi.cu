@@ -217,21 +217,31 @@ int eulernet::run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp,
 
 namespace {
 
+// A device array of at least `need` entries.  A failed allocation leaves it
+// empty with no capacity, so that no later call takes it for the former one.
+template <class T>
+int grow(T** p, size_t* cap, size_t need) {
+  if (need <= *cap && *p) return EULER_OK;
+  cudaFree(*p);
+  *p = nullptr;
+  *cap = 0;
+  CUDA_TRY(cudaMalloc(p, sizeof(T) * std::max<size_t>(need, 1)));
+  *cap = need;
+  return EULER_OK;
+}
+
 int refresh_step_tables(euler_net* h, double dt, double T, cudaStream_t s) {
   const int64_t K = euler_num_steps(dt, T);
   if (h->c_dt == dt && h->c_T == T) return EULER_OK;
+  h->c_dt = h->c_T = -1.0;  // a failure part way leaves neither the old tables nor the new ones
+  int rc;
   std::vector<float4> p0(h->n);
   std::vector<float> muh(h->n);
   step_p0(*h, dt, 0, h->n, p0.data(), muh.data());
   if (h->sv_len > 0) {
     std::vector<int32_t> mt((size_t)K * h->n);
     step_servers(*h, dt, 1, K, mt.data());
-    if (mt.size() > h->mtab_cap || !h->d_mtab) {
-      cudaFree(h->d_mtab);
-      h->d_mtab = nullptr;
-      CUDA_TRY(cudaMalloc(&h->d_mtab, sizeof(int32_t) * mt.size()));
-      h->mtab_cap = mt.size();
-    }
+    if ((rc = grow(&h->d_mtab, &h->mtab_cap, mt.size()))) return rc;
     CUDA_TRY(cudaMemcpyAsync(h->d_mtab, mt.data(), sizeof(int32_t) * mt.size(), cudaMemcpyHostToDevice, s));
     CUDA_TRY(cudaStreamSynchronize(s));
     h->h2d_bytes += (int64_t)(sizeof(int32_t) * mt.size());
@@ -242,12 +252,7 @@ int refresh_step_tables(euler_net* h, double dt, double T, cudaStream_t s) {
   std::vector<float> lam((size_t)K * std::max(h->n_ex, 1), 0.0f);
   if (h->n_ex > 0) step_lam(*h, dt, 0, K * h->n_ex, lam.data());
   if (!h->d_p0) CUDA_TRY(cudaMalloc(&h->d_p0, sizeof(float4) * (size_t)h->n));
-  if (lam.size() > h->lam_cap) {
-    if (h->d_lam) CUDA_TRY(cudaFree(h->d_lam));
-    h->d_lam = nullptr;
-    CUDA_TRY(cudaMalloc(&h->d_lam, sizeof(float) * lam.size()));
-    h->lam_cap = lam.size();
-  }
+  if ((rc = grow(&h->d_lam, &h->lam_cap, lam.size()))) return rc;
   CUDA_TRY(cudaMemcpyAsync(h->d_p0, p0.data(), sizeof(float4) * p0.size(), cudaMemcpyHostToDevice, s));
   CUDA_TRY(cudaMemcpyAsync(h->d_lam, lam.data(), sizeof(float) * lam.size(), cudaMemcpyHostToDevice, s));
   h->h2d_bytes += (int64_t)(sizeof(float4) * p0.size() + sizeof(float) * lam.size());
@@ -439,13 +444,14 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
 
 int ensure_hbm_state(euler_net* h, int64_t R) {
   const int64_t ld = hbm_ld(R);
-  if (ld <= h->hbm_cap_ld && R <= h->hbm_cap_R && h->d_N) return EULER_OK;
+  if (ld <= h->hbm_cap_ld && R <= h->hbm_cap_R) return EULER_OK;
   cudaFree(h->d_N);
   cudaFree(h->d_Redge);
   cudaFree(h->d_racc);
   h->d_N = nullptr;
   h->d_Redge = nullptr;
   h->d_racc = nullptr;
+  h->hbm_cap_ld = h->hbm_cap_R = 0;
   CUDA_TRY(cudaMalloc(&h->d_N, sizeof(int32_t) * (size_t)h->n * ld));
   CUDA_TRY(cudaMalloc(&h->d_Redge,
                       sizeof(int32_t) * (size_t)std::max(h->hbm_depth, 2) * std::max(h->E, 1) * ld));
@@ -885,16 +891,6 @@ int euler_net_plan(euler_net* h, int32_t scheme, int64_t R, int32_t* form, int32
 
 namespace {
 
-template <class T>
-int grow(T** p, size_t* cap, size_t need) {
-  if (need <= *cap && *p) return EULER_OK;
-  cudaFree(*p);
-  *p = nullptr;
-  CUDA_TRY(cudaMalloc(p, sizeof(T) * std::max<size_t>(need, 1)));
-  *cap = need;
-  return EULER_OK;
-}
-
 // The run parameters of a plain simulation call (tables current for dt).
 RunParams simulate_params(const euler_net* h, int32_t scheme, double dt, int64_t K, int64_t R, uint64_t seed,
                           int64_t rep_begin, int64_t* stats, int32_t tile_reps, int64_t num_tiles) {
@@ -993,6 +989,7 @@ namespace {
 
 int refresh_grad_tables(euler_net* h, double dt, double T, cudaStream_t s) {
   if (h->g_dt == dt && h->g_T == T) return EULER_OK;
+  h->g_dt = h->g_T = -1.0;
   const int64_t K = euler_num_steps(dt, T);
   std::vector<float> p0f(h->n);
   for (int32_t i = 0; i < h->n; ++i) p0f[i] = -fm::expm1(-(float)(h->mu[i] * dt));
@@ -1157,12 +1154,13 @@ int euler_net_simulate_average(euler_net* h, double dt, double T, int64_t R, uin
   if (!h || !stats_avg || R < 0) return fail(EULER_ERR_ARG, "bad average-scheme arguments");
   const size_t len = (size_t)euler_stats_len(h->n, R);
   if (!stats_b || !stats_f) {
-    if (len > h->avg_cap || !h->d_avg_b) {
+    if (len > h->avg_cap) {
       cudaFree(h->d_avg_b);
       cudaFree(h->d_avg_f);
       h->d_avg_b = h->d_avg_f = nullptr;
-      CUDA_TRY(cudaMalloc(&h->d_avg_b, sizeof(int64_t) * std::max<size_t>(len, 1)));
-      CUDA_TRY(cudaMalloc(&h->d_avg_f, sizeof(int64_t) * std::max<size_t>(len, 1)));
+      h->avg_cap = 0;
+      CUDA_TRY(cudaMalloc(&h->d_avg_b, sizeof(int64_t) * len));
+      CUDA_TRY(cudaMalloc(&h->d_avg_f, sizeof(int64_t) * len));
       h->avg_cap = len;
     }
     if (!stats_b) stats_b = h->d_avg_b;

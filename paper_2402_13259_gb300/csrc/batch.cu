@@ -47,7 +47,8 @@ struct euler_batch {
   int hbm_block = kHbmBlock;
   int hbm_graph_steps = 32;
   int rt_shift = 0;  // persistent tiles scaled by 2^rt_shift
-  // current plan
+  // current plan (planned: complete; a re-planning that failed leaves none)
+  bool planned = false;
   int block = 256;
   int64_t smem_cap = 0;  // shared-memory budget per CTA used by the plan
   int grid = 0;
@@ -141,6 +142,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
                     double cp_factor) {
   if (block % 32 || block < 32 || block > 512) return bfail(EULER_ERR_ARG, "batch block must be a multiple of 32 in [32, 512]");
   cap = std::min<int64_t>(cap, b->smem_optin);
+  b->planned = false;
   b->block = block;
   b->smem_cap = cap;
   b->rt_shift = rt_shift;
@@ -255,6 +257,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
   if ((size_t)b->num_items > b->items_cap) {
     cudaFree(b->d_items);
     b->d_items = nullptr;
+    b->items_cap = 0;
     BTRY(cudaMalloc(&b->d_items, sizeof(int2) * std::max(b->num_items, 1)));
     b->items_cap = b->num_items;
   }
@@ -262,6 +265,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
   if (sacc_need > b->sacc_cap) {
     cudaFree(b->d_sacc);
     b->d_sacc = nullptr;
+    b->sacc_cap = 0;
     BTRY(cudaMalloc(&b->d_sacc, sizeof(unsigned long long) * sacc_need));
     b->sacc_cap = sacc_need;
   }
@@ -275,6 +279,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
   if (alone_need > b->alone_cap) {
     cudaFree(b->d_alone);
     b->d_alone = nullptr;
+    b->alone_cap = 0;
     BTRY(cudaMalloc(&b->d_alone, sizeof(unsigned long long) * alone_need));
     b->alone_cap = alone_need;
   }
@@ -286,6 +291,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
     b->exec = nullptr;
   }
   b->graph_stats.clear();
+  b->planned = true;
   return EULER_OK;
 }
 
@@ -550,6 +556,7 @@ int euler_batch_run(euler_batch* b, int64_t* const* stats, void* cuda_stream) tr
   if (!b || (b->count > 0 && !stats)) return bfail(EULER_ERR_ARG, "bad batch run arguments");
   for (int j = 0; j < b->count; ++j)
     if (!stats[j]) return bfail(EULER_ERR_ARG, "a stats pointer is NULL");
+  if (!b->planned) return bfail(EULER_ERR_OOM, "the batch has no plan: its last re-planning failed");
   cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
   // the handles' per-step tables for the batch's (dt, T): another call on a
   // handle since the plan may have rebuilt them elsewhere

@@ -114,3 +114,73 @@ bad = sorted(set(x for x in t.splitlines() if "VIOLATION" in x))
 assert not bad, bad[:6]
 h.close()
 ''')
+
+
+@pytest.mark.parametrize("call", ["simulate", "sojourn", "grad", "average"])
+@pytest.mark.parametrize("form", [1, 2])
+def test_calls_after_a_failed_allocation(host, call, form):
+    """A call whose n-th allocation fails returns an error; the next, smaller
+    call on the handle runs on allocations that hold what it addresses."""
+    host(f'''
+def average(h, scheme, R, T=1.0):
+    a = dev(8 * Bd.stats_len(h.n, R))
+    rc = L.euler_net_simulate_average(h._h, 0.1, T, R, 1, 0, a, None, None, None)
+    RT.cudaFree(a)
+    return rc
+def go(h, R, T):
+    call = {call!r}
+    return (simulate(h, 0, R, T=T) if call == "simulate" else sojourn(h, 0, R, 5, T=T) if call == "sojourn" else
+            grad(h, 0, R, T=T) if call == "grad" else average(h, 0, R, T=T))
+real_dev = dev
+def dev(n):  # the test's own buffers never fail
+    F.fake_fail_malloc(0)
+    p = real_dev(n)
+    F.fake_fail_malloc(fail)
+    return p
+failed = 0
+for fail_at in range(1, 12):
+    h = net(chain(40, 3))
+    h.set_servers_schedule(np.full((3, 40), 4, np.int32), 0.3)
+    h.set_option(Bd.OPT_FORM, {form})
+    fail = 0
+    assert go(h, 300, 1.0) == 0
+    fail = fail_at
+    rc = go(h, 900, 2.0)
+    fail = 0
+    F.fake_fail_malloc(0)
+    failed += rc != 0
+    for R, T in ((200, 1.0), (900, 0.7), (100, 2.0), (900, 2.0)):
+        assert go(h, R, T) == 0, (fail_at, R)
+    h.close()
+bad = sorted(set(x for x in log().splitlines() if "VIOLATION" in x))
+assert not bad, bad[:6]
+assert failed > 0
+''')
+
+
+def test_batch_after_a_failed_allocation(host):
+    """A batch whose re-planning fails an allocation part way either reports it
+    or runs on allocations that hold what it addresses."""
+    host('''
+for fail_at in range(0, 12):
+    hs = [net(chain(n, 2)) for n in (3, 40, 120)]
+    runs = (Bd._Run * 3)(*[Bd._Run(j % 2, 0.1, 1.0 + j, R, 5, 0) for j, R in enumerate((20000, 5000, 2000))])
+    arr = (C.c_void_p * 3)(*[h._h for h in hs])
+    b = C.c_void_p()
+    assert L.euler_batch_create(C.byref(b), arr, runs, 3) == 0
+    st = [dev(8 * Bd.stats_len(h.n, r.replications)) for h, r in zip(hs, runs)]
+    ptr = (C.c_void_p * 3)(*[x.value for x in st])
+    F.fake_fail_malloc(fail_at)
+    L.euler_batch_autotune(b, None, None)
+    F.fake_fail_malloc(0)
+    L.euler_batch_run(b, ptr, None)
+    L.euler_batch_destroy(b)
+    for h in hs:
+        h.close()
+    for x in st:
+        RT.cudaFree(x)
+t = log()
+assert "batch_kernel" in t
+bad = sorted(set(x for x in t.splitlines() if "VIOLATION" in x))
+assert not bad, bad[:6]
+''')
