@@ -283,9 +283,9 @@ int eulernet::prepare_step_tables(euler_net* h, double dt, double T, cudaStream_
 // 1.9 tasks 20.8 ms listed, 24.3 ms in place).
 //
 // Returns false if not even one replication fits a tile.
-bool eulernet::plan_slots(const euler_net* h, int64_t R, bool grad, int32_t soj, int force_Rt, int force_block,
-                          SlotPlan* sp) {
-  const int32_t ring = h->tables().ring;
+bool eulernet::plan_slots(const euler_net* h, int32_t scheme, int64_t R, bool grad, int32_t soj, int force_Rt,
+                          int force_block, SlotPlan* sp) {
+  const int32_t ring = h->slot_ring(scheme);
   auto bytes = [&](int64_t Rt) { return slot_smem_bytes(h->n, h->E, ring, h->n_ex, Rt, grad, soj); };
   const int64_t limit = h->smem_optin;
   const int64_t per_rep = (bytes(33) - bytes(1)) / 32;
@@ -335,8 +335,8 @@ bool eulernet::hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp
   return (int64_t)h->n * R >= kHbmMinUnitsPerStep && sp.fill < kTileMinFill;
 }
 
-bool eulernet::plan_alone(const euler_net* h, int64_t R, SlotPlan* sp) {
-  return plan_slots(h, R, false, 0, 0, 0, sp) && !hbm_beats_tiles(h, R, *sp);
+bool eulernet::plan_alone(const euler_net* h, int32_t scheme, int64_t R, SlotPlan* sp) {
+  return plan_slots(h, scheme, R, false, 0, 0, 0, sp) && !hbm_beats_tiles(h, R, *sp);
 }
 
 namespace {
@@ -409,7 +409,7 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
   SlotPlan sp;
   if (pl->form == 1) {
     const int block = h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : 0;
-    const bool tiled = plan_slots(h, R, false, 0, Rt, block, &sp);
+    const bool tiled = plan_slots(h, scheme, R, false, 0, Rt, block, &sp);
     if (!tiled && forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "network tile does not fit in shared memory");
     const bool large = forced_form <= 0 && (int64_t)h->n * R >= kHbmMinUnitsPerStep;
     const bool bad_block = block > 0 && (block % 32 || (Rt > 0 && block % Rt) || block > (large ? 256 : 512));
@@ -937,7 +937,7 @@ int eulernet::simulate_alone(euler_net* h, int32_t scheme, double dt, double T, 
   if (R == 0) return EULER_OK;
   RunParams p = simulate_params(h, scheme, dt, K, R, seed, rep_begin, stats, 32, (R + 31) / 32);
   SlotPlan sp;
-  if (acc && plan_alone(h, R, &sp)) {
+  if (acc && plan_alone(h, scheme, R, &sp)) {
     p.acc = acc;
     return run_slots(h, p, kSlotPlain, sp, (int)std::min<int64_t>(h->sm_count, sp.tiles), s);
   }
@@ -1065,7 +1065,7 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   // station and replication in global memory, in the same step order).
   const int forced = (int)h->opt[EULER_OPT_FORM];
   SlotPlan sp;
-  const bool tiled = plan_slots(h, R, true, 0, 0, 0, &sp);
+  const bool tiled = plan_slots(h, scheme, R, true, 0, 0, 0, &sp);
   if (forced == 2 || (forced <= 0 && (tiled ? hbm_beats_tiles(h, R, sp) : (int64_t)h->n * R >= kHbmMinUnitsPerStep))) {
     const int64_t ld = hbm_ld(R);
     rc = grow(&h->d_gmu, &h->gmu_cap, (size_t)(h->n * ld));

@@ -102,9 +102,9 @@ int64_t pow2_floor(int64_t v) {
   return p;
 }
 
-// Shared memory of network j's tile of Rt replications.
-int64_t tile_bytes(const euler_net* h, int64_t Rt) {
-  return slot_smem_bytes(h->n, h->E, h->tables().ring, h->n_ex, Rt, false, 0);
+// Shared memory of a network's tile of Rt replications.
+int64_t tile_bytes(const euler_net* h, int32_t scheme, int64_t Rt) {
+  return slot_smem_bytes(h->n, h->E, h->slot_ring(scheme), h->n_ex, Rt, false, 0);
 }
 
 bool runs_hbm(const euler_batch* b, int j) { return b->is_hbm[j] != 0; }
@@ -119,7 +119,7 @@ bool tile_for(const euler_batch* b, int j, int block, int64_t cap, int rt_shift,
   Rt = rt_shift >= 0 ? Rt << rt_shift : Rt >> -rt_shift;
   Rt = std::max<int64_t>(1, std::min<int64_t>(Rt, block));
   for (; Rt >= 1; Rt /= 2)
-    if (tile_bytes(h, Rt) <= cap) {
+    if (tile_bytes(h, b->runs[j].scheme, Rt) <= cap) {
       *Rt_out = Rt;
       return true;
     }
@@ -167,7 +167,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
       for (int j = 0; j < b->count; ++j) {
         if (b->is_hbm[j]) continue;
         const euler_net* h = b->nets[j];
-        smem = std::max<int64_t>(smem, tile_bytes(h, Rt_of[j]));
+        smem = std::max<int64_t>(smem, tile_bytes(h, b->runs[j].scheme, Rt_of[j]));
         work += (double)h->n * (double)euler_num_steps(b->runs[j].dt, b->runs[j].T) * (double)b->runs[j].replications;
         n_items += (double)((b->runs[j].replications + Rt_of[j] - 1) / Rt_of[j]);
       }
@@ -203,7 +203,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
       continue;
     }
     const int64_t Rt = Rt_of[j];
-    smem = std::max<int64_t>(smem, tile_bytes(h, Rt));
+    smem = std::max<int64_t>(smem, tile_bytes(h, r.scheme, Rt));
     slot = std::max<int64_t>(slot, slot_acc_len(h->n, h->n_ex, Rt));
     RunParams p;
     std::memset(&p, 0, sizeof p);
@@ -273,7 +273,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
   for (int j : b->hbm_nets) {
     const euler_net* h = b->nets[j];
     SlotPlan sp;
-    if (plan_alone(h, b->runs[j].replications, &sp))
+    if (plan_alone(h, b->runs[j].scheme, b->runs[j].replications, &sp))
       alone_need = std::max(alone_need, (size_t)(slot_acc_len(h->n, h->n_ex, sp.Rt) * std::min<int64_t>(h->sm_count, sp.tiles)));
   }
   if (alone_need > b->alone_cap) {
@@ -409,7 +409,7 @@ int euler_batch_create(euler_batch** out, euler_net* const* nets, const euler_ru
   // 110 KiB where a network's smallest tile needs it.
   int64_t cap = 72 * 1024;
   for (int j = 0; j < count; ++j)
-    if ((int64_t)nets[j]->n * runs[j].replications < kHbmMinUnitsPerStep && tile_bytes(nets[j], 1) > cap) cap = 110 * 1024;
+    if ((int64_t)nets[j]->n * runs[j].replications < kHbmMinUnitsPerStep && tile_bytes(nets[j], runs[j].scheme, 1) > cap) cap = 110 * 1024;
   int rc = make_batch_plan(b, 512, cap, 0, kHbmMinUnitsPerStep, 1.0);
   if (rc) {
     euler_batch_destroy(b);

@@ -104,6 +104,12 @@ struct euler_net {
   int32_t dep_mode() const { return opt[EULER_OPT_DEPARTURE] > 0 ? (int32_t)opt[EULER_OPT_DEPARTURE] : 0; }
   const int32_t* mtab() const { return sv_len > 0 ? d_mtab : nullptr; }
 
+  // Ring slots of routed counts in a tile of the persistent form: a backward
+  // slot reads only the one before it.
+  int32_t slot_ring(int32_t scheme) const {
+    return scheme == EULER_BACKWARD || hbm_depth < 2 ? 2 : hbm_depth;
+  }
+
   eulernet::NetTables tables() const {
     eulernet::NetTables t;
     t.n = n;
@@ -121,7 +127,7 @@ struct euler_net {
     t.n_ex = n_ex;
     t.pos_level = d_pos_level;
     t.rec = d_rec;
-    t.ring = hbm_depth > 2 ? hbm_depth : 2;
+    t.ring = slot_ring(EULER_FORWARD);
     return t;
   }
 };
@@ -168,13 +174,13 @@ struct SlotPlan {
   int64_t smem = 0, tiles = 0;
   double fill = 1.0;      // share of the SMs' replication slots in use
 };
-bool plan_slots(const euler_net* h, int64_t R, bool grad, int32_t soj, int force_Rt, int force_block, SlotPlan* sp);
+bool plan_slots(const euler_net* h, int32_t scheme, int64_t R, bool grad, int32_t soj, int force_Rt, int force_block, SlotPlan* sp);
 bool hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp);
 int run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp, int grid, cudaStream_t s);
 
 // Whether a plain run of R replications takes the persistent form, with *sp
 // its plan, or the HBM form.
-bool plan_alone(const euler_net* h, int64_t R, SlotPlan* sp);
+bool plan_alone(const euler_net* h, int32_t scheme, int64_t R, SlotPlan* sp);
 
 // A plain simulation call of a network that fills the GPU by itself (the
 // batched form's large networks), in the form of plan_alone: tables made

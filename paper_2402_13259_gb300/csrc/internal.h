@@ -29,8 +29,8 @@ struct NetTables {
   // 2, level % ring, position of in-edge 3 in in_edge, in-edges beyond three};
   // an in-edge that is not there is edge E, whose row of counts is zero
   const int4* rec;
-  int32_t ring;                // routed-count ring slots of the slot schedules:
-                               // max(2, largest level gap of an edge + 1)
+  int32_t ring;                // routed-count ring slots of the forward slot
+                               // schedule: max(2, largest level gap of an edge + 1)
 };
 
 // Sojourn times (Algorithm 4): S tagged customers per replication enter

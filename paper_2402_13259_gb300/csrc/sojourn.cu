@@ -119,7 +119,7 @@ extern "C" int euler_net_sojourn(euler_net* h, int32_t scheme, double dt, double
   // lives in global memory and the warp of a customer's station advances it.
   const int forced = (int)h->opt[EULER_OPT_FORM];
   SlotPlan sp;
-  const bool tiled = plan_slots(h, R, false, samples, 0, 0, &sp);
+  const bool tiled = plan_slots(h, scheme, R, false, samples, 0, 0, &sp);
   const bool large = (int64_t)h->n * R >= kHbmMinUnitsPerStep;
   // a network and sample count beyond a tile of one replication (its state,
   // one step's inputs and departures, its customers), unless the HBM form is

@@ -61,9 +61,9 @@ namespace eulernet {
 // Dynamic shared memory of the slot kernels (see slot_smem_bytes), addressed
 // by 32-bit word offsets: 1/k table [64] | counters [16] | racc i64 [Rt][4],
 // the replications' sums at the tile's end | N u32 [n][Rt], the state |
-// R i32 [ring][E+1][Rt], routed counts, row E zero (stands in for an in-edge
-// that is not there) | aex i32 [n_ex][Rt], this slot's arrivals of listed units
-// (backward) | list u16 [n Rt] | GRAD: mu_acc f64 [n][Rt], th_acc f64
+// R i32 [ring][E+1][Rt], routed counts (two ring slots backward, t.ring forward),
+// row E zero (stands in for an in-edge that is not there) | aex i32 [n_ex][Rt],
+// this slot's arrivals of listed units (backward) | list u16 [n Rt] | GRAD: mu_acc f64 [n][Rt], th_acc f64
 // [n_ex][Rt][3], score sums | SOJ: tagged customers' words u64, places i32 and
 // step counts i32, [S][Rt] each.
 extern __shared__ __align__(16) uint32_t slot_smem[];
@@ -105,8 +105,9 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
   const uint32_t rep0 = (uint32_t)(p.rep_begin + r0);
   // word offsets of the area
+  const int ring = SCHEME == 0 ? 2 : t.ring;
   const int ring_stride = (t.E + 1) * Rt;
-  const int oRacc = 80, oN = oRacc + 8 * Rt, oR = oN + U, oAex = oR + t.ring * ring_stride;
+  const int oRacc = 80, oN = oRacc + 8 * Rt, oR = oN + U, oAex = oR + ring * ring_stride;
   const int oList = oAex + t.n_ex * Rt, oMu = (oList + (U + 1) / 2 + 3) / 4 * 4;
   int* const ctr = reinterpret_cast<int*>(slot_smem + 64);
   uint16_t* const list = reinterpret_cast<uint16_t*>(slot_smem + oList);
@@ -127,7 +128,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
     const int pos = Rt > 1 ? (int)__umulhi((uint32_t)q, magic) : q;
     slot_smem[oN + q] = t.N0 ? (uint32_t)__ldg(t.N0 + __ldg(t.rec + 3 * pos).x) : 0u;
   }
-  for (int k = tid; k < t.ring * Rt; k += nthr) slot_smem[oR + (k / Rt) * ring_stride + t.E * Rt + k % Rt] = 0u;
+  for (int k = tid; k < ring * Rt; k += nthr) slot_smem[oR + (k / Rt) * ring_stride + t.E * Rt + k % Rt] = 0u;
   for (int k = tid; k < 8 * Rt; k += nthr) slot_smem[oRacc + k] = 0u;
   for (int k = tid; k < 4 * U + t.n_ex * Rt; k += nthr) __stcg(acc + k, 0ull);
   if (SOJ)
@@ -166,7 +167,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
     nres = slot_smem[oN + q];
   }
   for (int slot = 1; slot <= last; ++slot) {
-    mod_ring = mod_ring + 1 == t.ring ? 0 : mod_ring + 1;
+    mod_ring = mod_ring + 1 == ring ? 0 : mod_ring + 1;
     mod3 = mod3 == 2 ? 0 : mod3 + 1;
     int* const count = ctr + 4 + mod3;
     if (!RES && tid == 0) {
@@ -199,7 +200,7 @@ __device__ __forceinline__ void tile_slots(const NetTables& t, const RunParams& 
           } else {
             tau = slot - ra.y;
             const int rs = mod_ring - rc.y;
-            ocur = oR + (rs < 0 ? rs + t.ring : rs) * ring_stride;
+            ocur = oR + (rs < 0 ? rs + ring : rs) * ring_stride;
             act = tau >= 1 && tau <= p.K;
           }
           const bool draws = tau <= p.K;

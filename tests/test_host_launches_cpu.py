@@ -49,6 +49,16 @@ def chain(n, skip=1, lam=12.0, m=9, every=3):
     w = np.zeros(n); w[::every] = lam
     return W.Network(n, rp, col, prob, np.full(n, m), np.full(n, 1.1),
                      W.Arrivals(kind=W.ARR_SINUSOID, w=w, a=1.0, b=0.2, period=3.0, phase=0.1))
+def dag(n, edges, every=4):
+    rp, col, prob = W.csr_from_edges(n, edges)
+    w = np.zeros(n); w[::every] = 6.0
+    return W.Network(n, rp, col, prob, np.full(n, 9), np.full(n, 1.1),
+                     W.Arrivals(kind=W.ARR_SINUSOID, w=w, a=1.0, b=0.2, period=3.0, phase=0.1))
+def complete(n):
+    return dag(n, [(i, j, 0.9 / (n - 1 - i)) for i in range(n) for j in range(i + 1, n)])
+def two_wide(levels):  # two stations to a level, one edge from the first to the last
+    e = [(2 * l + a, 2 * l + 2 + b, 0.4) for l in range(levels - 1) for a in range(2) for b in range(2)]
+    return dag(2 * levels, e + [(0, 2 * levels - 1, 0.1)])
 def net(x):
     return Bd.EulerNet(x)
 def simulate(h, scheme, R, dt=0.1, T=1.0):
@@ -184,3 +194,18 @@ assert "batch_kernel" in t
 bad = sorted(set(x for x in t.splitlines() if "VIOLATION" in x))
 assert not bad, bad[:6]
 ''')
+
+
+def test_backward_tiles_hold_two_ring_slots(host):
+    """A backward slot reads the slot before it only, so long edges take no
+    replications from a backward tile; the bytes fit what the kernel addresses."""
+    host("""
+for make, least in ((lambda: complete(40), 33), (lambda: two_wide(100), 33), (lambda: chain(20, 19), 250)):
+    h = net(make())
+    h.set_option(Bd.OPT_FORM, 1)
+    b, f = h.plan(0, 500_000), h.plan(1, 500_000)
+    assert b["form"] == f["form"] == 1
+    assert b["tile_reps"] >= least and b["tile_reps"] > 3 * f["tile_reps"], (b, f)
+    assert b["smem"] <= 227 * 1024
+    h.close()
+""")
