@@ -357,9 +357,11 @@ EULERNET_API int euler_net_status(euler_net* net, void* cuda_stream);
  * default.  Returns EULER_OK or EULER_ERR_ARG. */
 enum {
   EULER_OPT_FORM = 0,        /* 0 = auto (1, except 2 when a tile does not fit
-                                in shared memory, or when n x replications
+                                in shared memory; when n x replications
                                 >= 2^18 and whole tiles would leave a tenth
-                                of the SMs' room idle), 1 = persistent
+                                of the SMs' room idle or hold too few units,
+                                some hundreds; or for up to 6 replications of
+                                several thousand stations), 1 = persistent
                                 shared-memory kernel with block barriers, 2 = per-step
                                 kernels over HBM state replayed from a CUDA
                                 graph (forward scheme: one skewed launch per

@@ -321,7 +321,9 @@ bool eulernet::plan_slots(const euler_net* h, int32_t scheme, int64_t R, bool gr
   sp->block = force_block > 0 ? force_block : (int)(32 * std::max<int64_t>(1, std::min<int64_t>(kSlotThreads / 32, tasks)));
   sp->in_place = draws_in_place(tasks, sp->block / 32);
   sp->resident = tasks <= sp->block / 32 && soj == 0 && (!grad || sp->block <= kSlotResGradThreads);
-  sp->fill = (double)R / (double)(Rt * SM * waves_of(Rt));
+  sp->waves = waves_of(Rt);
+  sp->customers = soj;
+  sp->fill = (double)R / (double)(Rt * SM * sp->waves);
   return true;
 }
 
@@ -331,12 +333,46 @@ bool eulernet::plan_slots(const euler_net* h, int32_t scheme, int64_t R, bool gr
 // whole GPU (n R >= 2^18) the tiles' coarseness decides: with every SM's
 // replication slots in use the persistent form is 1.1 (2,000 stations,
 // s = 10 .. 10,000) to 1.6 times (100 stations) as fast.
-bool eulernet::hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp) {
-  return (int64_t)h->n * R >= kHbmMinUnitsPerStep && sp.fill < kTileMinFill;
+//
+// Unless its tiles are too small: where edges over many levels (a deep ring of
+// routed counts, forward) or many tagged customers leave a tile few units, a
+// slot is one unit's latency, paid once per wave of tiles.  Persistent over HBM
+// time: 70 units 5.2 to 6.5 (35 stations, every edge), 175 2.8, 300 1.2 to 1.5,
+// 342 1.09, 495 to 600 0.62 to 0.89.  With more than 128 customers their loop
+// takes most of a slot in both forms and the line moves down: 100 units 1.06 to
+// 1.9, 200 0.75 to 0.84 with 2,000 units of all replications to an SM and 1.08
+// to 1.5 with 6,600 to 13,000, 300 0.76 to 1.01.
+// `alone`: a network of a batch that its planner took out of the shared launch
+// may have fewer units a step; then four waves are needed (2 1.1 to 1.3, 4 1.1
+// to 2.1, one 0.4 to 0.7).
+//
+// And up to six replications of a network too large for the form with its
+// station sums in shared memory (48 bytes a station, some 3,400 stations): a
+// CTA per replication leaves the other SMs idle (3,500 to 9,000 stations: one
+// replication 1.9 to 3.9 times the HBM form's time, four 1.4 to 1.8, six 1.2,
+// eight 0.7 to 1.05).
+bool eulernet::hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp, bool alone) {
+  const int64_t units = (int64_t)h->n * R;
+  const bool large = units >= kHbmMinUnitsPerStep;
+  if (large && sp.fill < kTileMinFill) return true;
+  const int64_t least = sp.customers <= 128 ? 400 : units >= 2 * kHbmMinUnitsPerStep ? 250 : 150;
+  if ((large || alone) && sp.waves >= 4 && (int64_t)h->n * sp.Rt < least) return true;
+  return !large && R <= kFewReps &&
+         288 + 52 * (int64_t)h->n + 4 * (int64_t)h->tables().ring * h->E > h->smem_optin;
+}
+
+bool eulernet::takes_hbm(const euler_net* h, int64_t R, const SlotPlan& sp, cudaStream_t s) {
+  if (!hbm_beats_tiles(h, R, sp)) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return cs == cudaStreamCaptureStatusNone;
 }
 
 bool eulernet::plan_alone(const euler_net* h, int32_t scheme, int64_t R, SlotPlan* sp) {
-  return plan_slots(h, scheme, R, false, 0, 0, 0, sp) && !hbm_beats_tiles(h, R, *sp);
+  return plan_slots(h, scheme, R, false, 0, 0, 0, sp) && !hbm_beats_tiles(h, R, *sp, true);
 }
 
 namespace {
@@ -373,7 +409,8 @@ bool make_pipe_plan(const euler_net* h, int W, PipePlan* pp) {
 bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
 
 
-int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
+// The launch of a plain call on stream s.
+int make_plan(euler_net* h, int32_t scheme, int64_t R, cudaStream_t s, Plan* pl) {
   const int64_t limit = h->smem_optin;
   const int forced_form = (int)h->opt[EULER_OPT_FORM];
   int Rt = 0;  // 0: the planner's choice
@@ -413,7 +450,9 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, Plan* pl) {
     if (!tiled && forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "network tile does not fit in shared memory");
     const bool large = forced_form <= 0 && (int64_t)h->n * R >= kHbmMinUnitsPerStep;
     const bool bad_block = block > 0 && (block % 32 || (Rt > 0 && block % Rt) || block > (large ? 256 : 512));
-    if (!tiled || (forced_form <= 0 && hbm_beats_tiles(h, R, sp)) || (large && bad_block)) pl->form = 2;
+    // a block that only the persistent form takes keeps a smaller call in it
+    const bool hbm = forced_form <= 0 && (large || block <= 256) && takes_hbm(h, R, sp, s);
+    if (!tiled || hbm || (large && bad_block)) pl->form = 2;
     else if (bad_block) return fail(EULER_ERR_ARG, "block must be a multiple of 32 and of the tile, <= 512");
   }
   if (pl->form == 2) {
@@ -873,7 +912,7 @@ int euler_net_plan(euler_net* h, int32_t scheme, int64_t R, int32_t* form, int32
                    int32_t* block, int32_t* grid, int32_t* smem_bytes) try {
   if (!h || R < 1) return fail(EULER_ERR_ARG, "bad plan arguments");
   Plan pl;
-  int rc = make_plan(h, scheme, R, &pl);
+  int rc = make_plan(h, scheme, R, nullptr, &pl);
   if (rc) return rc;
   if (form) *form = pl.form;
   if (tile_reps) *tile_reps = pl.tile_reps;
@@ -964,7 +1003,7 @@ int euler_net_simulate(euler_net* h, int32_t scheme, double dt, double T, int64_
   int rc = refresh_step_tables(h, dt, T, s);
   if (rc) return rc;
   Plan pl;
-  rc = make_plan(h, scheme, R, &pl);
+  rc = make_plan(h, scheme, R, s, &pl);
   if (rc) return rc;
   RunParams p = simulate_params(h, scheme, dt, K, R, seed, rep_begin, stats, pl.tile_reps, pl.num_tiles);
   const NetTables t = h->tables();
@@ -1066,7 +1105,7 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
   const int forced = (int)h->opt[EULER_OPT_FORM];
   SlotPlan sp;
   const bool tiled = plan_slots(h, scheme, R, true, 0, 0, 0, &sp);
-  if (forced == 2 || (forced <= 0 && (tiled ? hbm_beats_tiles(h, R, sp) : (int64_t)h->n * R >= kHbmMinUnitsPerStep))) {
+  if (forced == 2 || (forced <= 0 && (tiled ? takes_hbm(h, R, sp, s) : (int64_t)h->n * R >= kHbmMinUnitsPerStep))) {
     const int64_t ld = hbm_ld(R);
     rc = grow(&h->d_gmu, &h->gmu_cap, (size_t)(h->n * ld));
     if (rc) return rc;

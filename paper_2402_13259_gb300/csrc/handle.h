@@ -135,9 +135,11 @@ struct euler_net {
 namespace eulernet {
 // Units per step (n R) from which one step has work for the whole GPU, the
 // share of the SMs' replication slots in use below which the HBM form is then
-// faster than the persistent one, and the HBM form's default threads per block.
+// faster than the persistent one, the replications up to which it is faster on
+// the largest networks (see hbm_beats_tiles), and its default threads per block.
 constexpr int64_t kHbmMinUnitsPerStep = int64_t(1) << 18;
 constexpr double kTileMinFill = 0.9;
+constexpr int64_t kFewReps = 6;
 constexpr int kHbmBlock = 256;
 // Bytes of HBM-form state per replication chunk, so that a chunk stays in L2.
 constexpr int64_t kHbmL2Budget = int64_t(64) << 20;
@@ -173,9 +175,15 @@ struct SlotPlan {
   bool resident = false;  // and no more tasks than warps: the kernel's RES variant
   int64_t smem = 0, tiles = 0;
   double fill = 1.0;      // share of the SMs' replication slots in use
+  int64_t waves = 1;      // tiles an SM runs one after another
+  int32_t customers = 0;  // tagged customers per replication
 };
 bool plan_slots(const euler_net* h, int32_t scheme, int64_t R, bool grad, int32_t soj, int force_Rt, int force_block, SlotPlan* sp);
-bool hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp);
+bool hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp, bool alone = false);
+// Whether a call on stream s that could take either form takes the HBM form:
+// where that is faster, unless s is being captured (a launch of its graphs is no
+// operation of another graph; the persistent form's kernels are).
+bool takes_hbm(const euler_net* h, int64_t R, const SlotPlan& sp, cudaStream_t s);
 int run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp, int grid, cudaStream_t s);
 
 // Whether a plain run of R replications takes the persistent form, with *sp

@@ -127,7 +127,7 @@ extern "C" int euler_net_sojourn(euler_net* h, int32_t scheme, double dt, double
   const int64_t least = 288 + 60 * (int64_t)h->n + 4 * (int64_t)h->E + 12 * (int64_t)samples;
   if (forced != 2 && (forced > 0 || !large) && least > h->smem_optin)
     return fail(EULER_ERR_TOO_LARGE, "sojourn tile does not fit in shared memory");
-  if (forced == 2 || !tiled || (forced <= 0 && hbm_beats_tiles(h, R, sp))) {
+  if (forced == 2 || !tiled || (forced <= 0 && takes_hbm(h, R, sp, s))) {
     const int64_t ld = hbm_ld(R);
     const size_t need = (size_t)samples * (size_t)ld;
     if (need > h->cust_cap) {

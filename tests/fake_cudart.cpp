@@ -206,6 +206,12 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
   *g = (cudaGraph_t)0x20;
   return cudaSuccess;
 }
+bool capturing = false;
+void fake_capturing(int on) { capturing = on != 0; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* st) {
+  *st = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
 cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode*) { return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) {
   *e = (cudaGraphExec_t)0x30;

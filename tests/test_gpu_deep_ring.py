@@ -56,3 +56,30 @@ def test_deep_ring(Bd, orc, make, size, R, scheme):
     for r in (0, R // 2, R - 1):
         want = orc.simulate(net, scheme, 0.1, 1.5, 1, 17, rep_begin=3 + r)["rep"][0]
         assert np.array_equal(rp[r], want), r
+
+
+def _chain(n):
+    return _net(n, [(i, i + 1, 0.6) for i in range(n - 1)])
+
+
+@pytest.mark.parametrize("make,size,R", [(_two_wide, 100, 1400), (_chain, 4000, 1)])
+def test_captured_call(Bd, make, size, R):
+    """A call whose eager form is per-step kernels, captured by the caller and
+    replayed."""
+    import torch
+    net = make(size)
+    h = Bd.EulerNet(net)
+    try:
+        assert h.plan(1, R)["form"] == 2
+        want = h.simulate(1, 0.1, 1.0, R, 5).cpu().numpy()
+        stats = torch.empty(Bd.stats_len(net.n, R), dtype=torch.int64, device="cuda")
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            h.simulate(1, 0.1, 1.0, R, 5, stats=stats, check=False)
+        for _ in range(2):
+            stats.fill_(-1)
+            g.replay()
+            h.status()
+            assert np.array_equal(stats.cpu().numpy(), want)
+    finally:
+        h.close()

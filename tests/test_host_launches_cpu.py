@@ -209,3 +209,49 @@ for make, least in ((lambda: complete(40), 33), (lambda: two_wide(100), 33), (la
     assert b["smem"] <= 227 * 1024
     h.close()
 """)
+
+
+def test_form_rule(host):
+    """The planner's form where a tile holds few units: per-step kernels for
+    many waves of small tiles and for a few replications of a large network,
+    the persistent form for one wave, for tiles of a few hundred units and for
+    backward tiles of the same networks; batches follow for the networks they
+    run by themselves."""
+    host("""
+def form(x, scheme, R):
+    h = net(x); f = h.plan(scheme, R)["form"]; h.close(); return f
+for x, R in ((complete(40), 10000), (complete(20), 40000), (two_wide(100), 1400), (two_wide(100), 10000)):
+    assert form(x, 1, R) == 2 and form(x, 0, R) == 1, (x.n, R)
+assert form(complete(12), 1, 40000) == 1 and form(two_wide(35), 1, 40000) == 1
+assert form(chain(100), 0, 10000) == form(chain(100), 1, 10000) == 1
+for n, R, want in ((3800, 1, 1), (3900, 1, 2), (3900, 6, 2), (3900, 7, 1), (3900, 60, 1), (9000, 4, 2), (2000, 1, 1)):
+    assert form(chain(n), 0, R) == want, (n, R)
+# tagged customers: as many as leave a tile one replication
+h = net(chain(100)); h2 = net(two_wide(100))
+for hh, R, S, want in ((h, 3000, 10000, "hbm_phase_kernel"), (h, 3000, 4, "persistent_kernel"),
+                       (h, 3000, 5000, "persistent_kernel"), (h, 300, 10000, "persistent_kernel"),
+                       (h2, 1400, 4, "hbm_phase_kernel"), (h2, 400, 4, "persistent_kernel")):
+    log()
+    assert sojourn(hh, 1, R, S) == 0
+    assert want in forms(log()), (R, S)
+log(); assert grad(h2, 1, 5000) == 0 and "hbm_phase_kernel" in forms(log())
+assert grad(h2, 0, 5000) == 0 and "persistent_kernel" in forms(log())
+# a caller's capture takes kernels, not the launch of another graph
+for x, R in ((h2, 5000), (net(chain(4000)), 1)):
+    for on, want in ((0, "hbm_phase_kernel"), (1, "persistent_kernel"), (0, "hbm_phase_kernel")):
+        F.fake_capturing(on); log()
+        assert simulate(x, 1, R) == 0 and want in forms(log())
+h.close(); h2.close()
+# in a batch: fewer than 2^18 units a step, but a tile beyond the shared launch's budget
+hs = [net(chain(167, 155)), net(chain(3))]
+for R, want in ((1500, "hbm_phase_kernel"), (300, "persistent_kernel")):
+    runs = (Bd._Run * 2)(Bd._Run(1, 0.1, 1.0, R, 5, 0), Bd._Run(1, 0.1, 0.5, 80, 5, 0))
+    b = C.c_void_p()
+    assert L.euler_batch_create(C.byref(b), (C.c_void_p * 2)(*[x._h for x in hs]), runs, 2) == 0
+    st = [dev(8 * Bd.stats_len(x.n, r.replications)) for x, r in zip(hs, runs)]
+    log()
+    assert L.euler_batch_run(b, (C.c_void_p * 2)(*[x.value for x in st]), None) == 0
+    t = log()
+    assert forms(t)[:2] == ["batch_kernel", want] and "VIOLATION" not in t, (R, forms(t))
+    L.euler_batch_destroy(b)
+""")
