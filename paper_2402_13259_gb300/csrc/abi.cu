@@ -327,6 +327,14 @@ bool eulernet::plan_slots(const euler_net* h, int32_t scheme, int64_t R, bool gr
   return true;
 }
 
+// What a requested tile of Rt replications may take (EULER_OPT_TILE_REPS): its
+// state, its replications' sums and 48 bytes a station.  The tile itself has no
+// station sums but lists, arrivals and a zero row, so a large one within this
+// limit may need more than it; it is then halved until it fits.
+static int64_t tile_limit_bytes(const euler_net* h, int64_t Rt) {
+  return 256 + 48 * (int64_t)h->n + Rt * (32 + 4 * ((int64_t)h->n + (int64_t)h->slot_ring(EULER_FORWARD) * h->E));
+}
+
 // The persistent form runs a slot with one or two block barriers and no launch,
 // state and lists in shared memory; the HBM form's per-step launches spread
 // any replication count evenly over the GPU.  Where a step has work for the
@@ -357,8 +365,7 @@ bool eulernet::hbm_beats_tiles(const euler_net* h, int64_t R, const SlotPlan& sp
   if (large && sp.fill < kTileMinFill) return true;
   const int64_t least = sp.customers <= 128 ? 400 : units >= 2 * kHbmMinUnitsPerStep ? 250 : 150;
   if ((large || alone) && sp.waves >= 4 && (int64_t)h->n * sp.Rt < least) return true;
-  return !large && R <= kFewReps &&
-         288 + 52 * (int64_t)h->n + 4 * (int64_t)h->tables().ring * h->E > h->smem_optin;
+  return !large && R <= kFewReps && tile_limit_bytes(h, 1) > h->smem_optin;
 }
 
 bool eulernet::takes_hbm(const euler_net* h, int64_t R, const SlotPlan& sp, cudaStream_t s) {
@@ -446,7 +453,9 @@ int make_plan(euler_net* h, int32_t scheme, int64_t R, cudaStream_t s, Plan* pl)
   SlotPlan sp;
   if (pl->form == 1) {
     const int block = h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : 0;
-    const bool tiled = plan_slots(h, scheme, R, false, 0, Rt, block, &sp);
+    bool tiled = plan_slots(h, scheme, R, false, 0, Rt, block, &sp);
+    if (!tiled && Rt > 1 && tile_limit_bytes(h, Rt) <= limit)
+      for (int rt = Rt / 2; rt >= 1 && !tiled; rt /= 2) tiled = plan_slots(h, scheme, R, false, 0, rt, block, &sp);
     if (!tiled && forced_form == 1) return fail(EULER_ERR_TOO_LARGE, "network tile does not fit in shared memory");
     const bool large = forced_form <= 0 && (int64_t)h->n * R >= kHbmMinUnitsPerStep;
     const bool bad_block = block > 0 && (block % 32 || (Rt > 0 && block % Rt) || block > (large ? 256 : 512));
@@ -1135,16 +1144,17 @@ int euler_net_grad(euler_net* h, int32_t scheme, double dt, double T, int64_t R,
     p.muh = h->d_muh;
     p.dep_mode = 0;
     p.mtab = h->mtab();
-    Plan pl;
-    pl.form = 2;
-    pl.block = h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : kHbmBlock;
-    if (pl.block % 32 || pl.block > 256) return fail(EULER_ERR_ARG, "HBM-form block must be a multiple of 32 <= 256");
+    // EULER_OPT_BLOCK is for the calls that fill the GPU and those that ask for
+    // this form; the persistent form's gradients choose their own block
+    const bool own_block = forced == 2 || (int64_t)h->n * R >= kHbmMinUnitsPerStep;
+    const int block = own_block && h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : kHbmBlock;
+    if (block % 32 || block > 256) return fail(EULER_ERR_ARG, "HBM-form block must be a multiple of 32 <= 256");
     CUDA_TRY(cudaMemsetAsync(stats, 0, sizeof(int64_t) * (size_t)euler_stats_len(h->n, R), s));
     HbmExtra xg;
     xg.mode = kHbmGrad;
     xg.mu_acc = h->d_gmu;
     xg.th_acc = h->d_gth;
-    rc = run_hbm_form(h, h->tables(), p, pl.block, s, xg);
+    rc = run_hbm_form(h, h->tables(), p, block, s, xg);
     if (rc) return rc;
     cudaError_t e = launch_grad_reduce(h->n, R, dt, stats, scores, h->d_gpartial, grad, value, grad_var,
                                        h->opt[EULER_OPT_GRAD_CENTER] > 0, s);

@@ -143,7 +143,9 @@ extern "C" int euler_net_sojourn(euler_net* h, int32_t scheme, double dt, double
       if (e != cudaSuccess) return cuda_fail(e, "sojourn customer state");
       h->cust_cap = need;
     }
-    const int block = h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : kHbmBlock;
+    // EULER_OPT_BLOCK as for euler_net_grad
+    const bool own_block = forced == 2 || (forced <= 0 && large);
+    const int block = own_block && h->opt[EULER_OPT_BLOCK] > 0 ? (int)h->opt[EULER_OPT_BLOCK] : kHbmBlock;
     if (block % 32 || block > 256) return fail(EULER_ERR_ARG, "HBM-form block must be a multiple of 32 <= 256");
     p.tile_reps = 32;
     p.num_tiles = (R + 31) / 32;

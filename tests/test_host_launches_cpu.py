@@ -255,3 +255,35 @@ for R, want in ((1500, "hbm_phase_kernel"), (300, "persistent_kernel")):
     assert forms(t)[:2] == ["batch_kernel", want] and "VIOLATION" not in t, (R, forms(t))
     L.euler_batch_destroy(b)
 """)
+
+
+def test_options_that_no_longer_fit_the_tile(host):
+    """A requested tile within the documented limit runs although the tile's
+    lists and arrivals take more than the station sums did; a block for the
+    persistent form does not stop a small call whose tile does not fit."""
+    host("""
+for n, Rt, want in ((450, 32, 16), (535, 32, 16), (545, 32, None), (400, 32, 32), (1611, 8, 4), (900, 16, 8),
+                    (30, 512, 256), (23, 512, 512), (60, 512, None)):
+    h = net(chain(n, every=1))
+    h.set_option(Bd.OPT_FORM, 1)
+    h.set_option(Bd.OPT_TILE_REPS, Rt)
+    for scheme in (0, 1):
+        fits = 256 + 48 * n + Rt * (32 + 4 * (n + 2 * (n - 1))) <= 227 * 1024
+        assert fits == (want is not None), (n, Rt)
+        try:
+            p = h.plan(scheme, 1000)
+            assert p["form"] == 1 and p["tile_reps"] == want and p["smem"] <= 227 * 1024, (n, Rt, p)
+        except Bd.EulerError as e:
+            assert e.code == -7 and not fits, (n, Rt, str(e))
+    assert simulate(h, 0, 100) == (0 if fits else -7)
+    h.close()
+# a deep ring leaves no forward tile: the per-step kernels, at their own block
+h = net(complete(60)); h.set_option(Bd.OPT_BLOCK, 512)
+log(); assert sojourn(h, 1, 100, 4) == 0 and "hbm_phase_kernel" in forms(log())
+h.set_option(Bd.OPT_FORM, 2); assert sojourn(h, 1, 100, 4) == -1
+h.close()
+h = net(chain(4000)); h.set_option(Bd.OPT_BLOCK, 512)
+log(); assert grad(h, 0, 2) == 0
+assert h.plan(0, 2)["form"] == 1
+h.close()
+""")
