@@ -193,8 +193,10 @@ static int slot_scratch(euler_net* h, int grid, RunParams* p) {
 
 // The launches of a persistent-form run (see SlotPlan): p complete but for what
 // the plan decides (p.acc: the caller's per-unit sums, or nullptr for the
-// handle's).  One launch covers at most about 2e10 station-step updates
-// (about a second), a whole number of waves of tiles.
+// handle's).  A launch takes whole waves of tiles over the whole horizon, as
+// many as stay below 2e10 station-step updates (about 0.6 s) and at least one: a
+// long horizon is one launch however long (100 stations, 10,000 replications,
+// 100,000 steps: 1e11 updates, some 3 s).
 int eulernet::run_slots(euler_net* h, RunParams p, int mode, const SlotPlan& sp, int grid, cudaStream_t s) {
   p.tile_reps = sp.Rt;
   p.task_lanes = sp.lanes;

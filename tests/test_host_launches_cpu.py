@@ -287,3 +287,22 @@ log(); assert grad(h, 0, 2) == 0
 assert h.plan(0, 2)["form"] == 1
 h.close()
 """)
+
+
+def test_launches_of_tiles(host):
+    """A run beyond 2e10 updates is several launches of whole waves; one wave is
+    one launch however long its horizon."""
+    host("""
+import re
+for R, K in ((30000, 10000), (30000, 1000), (300000, 1000), (10000, 400000)):
+    h = net(chain(100))
+    p = h.plan(0, R)
+    tiles = -(-R // p["tile_reps"])
+    log()
+    assert simulate(h, 0, R, dt=0.01, T=0.01 * K) == 0
+    got = [int(x) for x in re.findall(r"tiles=([0-9]+)", log())]
+    per = p["grid"] * max(1, int(2e10 / (100.0 * p["tile_reps"] * K * p["grid"])))
+    assert sum(got) == tiles and max(got) <= per and len(got) == -(-tiles // per), (R, K, got, per)
+    assert (len(got) > 1) == (R * K * 100 > 2e10 and tiles > p["grid"]), (R, K, got)
+    h.close()
+""")
