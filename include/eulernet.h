@@ -113,8 +113,15 @@ EULERNET_API int64_t euler_stats_len(int32_t n, int64_t replications);
  * Asynchronous on cuda_stream.  Argument errors are returned synchronously;
  * device-side errors (EULER_ERR_SAMPLER_CAP, EULER_ERR_OVERFLOW) are latched
  * in the handle and returned by euler_net_status().  Calls on one handle must
- * not overlap on different streams (the handle's per-call tables and error
- * word are shared).  The handle caches the per-dt tables of its last call. */
+ * not overlap on different streams (the handle's per-call tables, scratch and
+ * error word are shared).  The handle caches the per-dt tables of its last call,
+ * and keeps the scratch of its largest call until euler_net_destroy: in the
+ * persistent form 8 (4n + external stations) bytes for each replication that runs
+ * at a time (33 MB for 100 stations and 10,000 replications; the first call of a
+ * larger size allocates), in the HBM form the state of a chunk of replications
+ * (see EULER_OPT_HBM_CHUNK).  A call under stream capture takes the persistent
+ * form where its tiles fit shared memory, given that the tables of its (dt, T)
+ * are current. */
 EULERNET_API int euler_net_simulate(euler_net* net, int32_t scheme, double dt, double T,
                        int64_t replications, uint64_t seed, int64_t rep_begin,
                        int64_t* stats, void* cuda_stream);
@@ -195,7 +202,8 @@ EULERNET_API double euler_net_select_dt(const euler_net* net, double alpha);
  * Sums over replications run in blocks of 32 (ascending), then over blocks in
  * ascending order, so results do not depend on the launch.  Asynchronous on
  * cuda_stream; EULER_ERR_TOO_LARGE when a tile with its score sums does not
- * fit in shared memory. */
+ * fit in shared memory and n x replications < 2^18 or EULER_OPT_FORM asks for a
+ * tile (the HBM form runs any size). */
 EULERNET_API int euler_net_grad(euler_net* net, int32_t scheme, double dt, double T,
                                 int64_t replications, uint64_t seed, int64_t rep_begin,
                                 double* grad, double* value, double* grad_var, double* scores,
@@ -273,8 +281,10 @@ EULERNET_API int euler_net_grad_coupled(euler_net* net, int32_t scheme, double d
  * step, rep_begin + r): the first uniform decides the stay, the second word
  * picks the departing customer.  Results do not depend on the launch.
  * Asynchronous on cuda_stream.  EULER_ERR_ARG for a station or tau0 out of
- * range or samples outside [1, 65536]; EULER_ERR_TOO_LARGE when a tile with
- * its customers does not fit in shared memory. */
+ * range or samples outside [1, 65536]; EULER_ERR_TOO_LARGE when n x replications
+ * < 2^18 and 288 + 60 n + 4 nnz + 12 samples exceeds the shared memory of a block
+ * (227 KB), unless EULER_OPT_FORM = 2; EULER_OPT_FORM = 1 at any size.  (This is the call's limit on small runs,
+ * whichever form would run them.) */
 EULERNET_API int euler_net_sojourn(euler_net* net, int32_t scheme, double dt, double T,
                                    int64_t replications, uint64_t seed, int64_t rep_begin,
                                    int32_t station, int64_t tau0, int32_t samples, int32_t* sojourn,
@@ -302,9 +312,11 @@ typedef struct euler_batch euler_batch; /* opaque */
  * these networks one after another; the others share one
  * persistent launch whose work items are (network, tile of replications),
  * ordered by decreasing cost, with per-network tile sizes that fill the
- * block.  Errors: EULER_ERR_ARG, EULER_ERR_TOO_LARGE (a network whose
- * smallest tile does not fit in shared memory), EULER_ERR_CUDA,
- * EULER_ERR_OOM. */
+ * block.  A network of the others whose tile does not fit the launch's
+ * shared-memory budget, or whose items would outlast the launch, runs by itself
+ * too.  Errors: EULER_ERR_ARG, EULER_ERR_TOO_LARGE (a network below the threshold
+ * with 288 + 4 (n + ring nnz) bytes, ring = max(2, largest level gap of an edge
+ * + 1), beyond the budget of 110 KiB), EULER_ERR_CUDA, EULER_ERR_OOM. */
 EULERNET_API int euler_batch_create(euler_batch** out, euler_net* const* nets,
                                     const euler_run* runs, int32_t count);
 
@@ -312,26 +324,29 @@ EULERNET_API int euler_batch_create(euler_batch** out, euler_net* const* nets,
  * persistent launch's threads per block (stations per CTA), shared-memory
  * budget per CTA and tile scale (replications per tile, x 1/2, 1, 2); the HBM
  * form's threads per step kernel and slots per graph replay (steps per
- * launch, 16 / 32 / 64), on up to six of its networks; then the n x
- * replications threshold between the two kinds (2^16, 2^18, 2^20 or none).
- * Synchronises `cuda_stream`; returns the persistent launch's block size in
- * *block_out (may be NULL). */
+ * launch, 16 / 32 / 64), on up to six of the networks run by themselves (those
+ * among them that take that form); then the n x replications threshold from
+ * which a network runs by itself (2^16, 2^18, 2^20 or none).  Synchronises
+ * `cuda_stream`; returns the persistent launch's block size in *block_out (may
+ * be NULL). */
 EULERNET_API int euler_batch_autotune(euler_batch* b, void* cuda_stream, int32_t* block_out);
 
 /* Run every request: stats[j] is run j's caller-owned DEVICE buffer of
  * euler_stats_len(n_j, R_j) int64, laid out as for euler_net_simulate.  The
  * persistent part (zeroing of every stats buffer plus one persistent kernel
  * per scheme) is captured once in a CUDA graph and replayed; a call with
- * other stats pointers re-captures.  The HBM-form networks follow on the
- * same stream, each replaying its own graph of per-step kernels.  Results
- * equal one euler_net_simulate call per request.  Asynchronous on
+ * other stats pointers re-captures.  The networks run by themselves follow on
+ * the same stream, one after another, each in the form euler_net_simulate would
+ * take.  After a failed re-planning (euler_batch_autotune out of memory) it
+ * returns EULER_ERR_OOM.  Results equal one euler_net_simulate call per request.  Asynchronous on
  * cuda_stream; device-side errors via euler_batch_status. */
 EULERNET_API int euler_batch_run(euler_batch* b, int64_t* const* stats, void* cuda_stream);
 
 /* The batch's current plan (after euler_batch_create, or the autotuner's
- * choice): *hbm_networks = requests run in the HBM form, *hbm_min_units =
- * their n x replications threshold (0: none), *critical_path = 1 if the
- * critical-path rule moves long work items to the HBM form, *block and
+ * choice): *hbm_networks = requests run by themselves (in the persistent or the
+ * HBM form), *hbm_min_units = their n x replications threshold (0: none),
+ * *critical_path = 1 if a network whose work items would outlast the shared
+ * launch runs by itself, *block and
  * *tile_shift = the persistent launch's threads per block and tile scale
  * (replications per tile x 2^tile_shift), *hbm_block and *graph_steps = the
  * HBM form's threads per step kernel and slots per graph replay.  Any output

@@ -2,7 +2,7 @@
 // persistent launch fed by a work queue, planned and autotuned on the host and
 // replayed from a CUDA graph.
 //
-// Two kinds of networks.  A network with n_j R_j >= hbm_min_units units per
+// Two kinds of networks.  A network with n_j R_j >= alone_min_units units per
 // step fills the GPU by itself: it runs as a euler_net_simulate call does, in
 // the persistent or the HBM form, one such network after another (64 mixed
 // networks 67.6 ms; with these in the HBM form 74.3 ms).  The others share one
@@ -12,13 +12,15 @@
 // Rt_j (a power of two) so that its widest phase keeps the block busy
 // (forward: widest level x Rt_j ~ block; backward: all stations), scaled by
 // 2^rt_shift, reduced until its tile's state fits the shared-memory budget;
-// its per-unit sums live in the CTA's slot of a global scratch array.  Items are sorted by decreasing cost n_j K_j Rt_j so the
-// last CTAs to finish take the cheapest items.
+// its per-unit sums live in the CTA's slot of a global scratch array.  Items are
+// sorted by decreasing cost n_j K_j Rt_j so the last CTAs to finish take the
+// cheapest items.
 //
 // The autotuner searches the persistent launch's threads per block (stations
 // per CTA), shared-memory budget and tile scale (replications per tile), the
 // HBM form's threads per block and slots per graph replay (steps per
-// launch), and the n R threshold between the two kinds.
+// launch, for the networks run by themselves that take it), and the n R
+// threshold between the two kinds.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -40,9 +42,9 @@ struct euler_batch {
   std::vector<euler_run> runs;
   int device = 0, sm_count = 0, smem_optin = 0;
   // networks run by themselves, and the HBM form's launch shape for those that take it
-  std::vector<int> hbm_nets;
-  std::vector<char> is_hbm;  // per network
-  int64_t hbm_min_units = kHbmMinUnitsPerStep;
+  std::vector<int> alone_nets;
+  std::vector<char> is_alone;  // per network
+  int64_t alone_min_units = kHbmMinUnitsPerStep;
   double cp_factor = 1.0;  // critical-path rule (see make_batch_plan); <= 0 off
   int hbm_block = kHbmBlock;
   int hbm_graph_steps = 32;
@@ -107,7 +109,7 @@ int64_t tile_bytes(const euler_net* h, int32_t scheme, int64_t Rt) {
   return slot_smem_bytes(h->n, h->E, h->slot_ring(scheme), h->n_ex, Rt, false, 0);
 }
 
-bool runs_hbm(const euler_batch* b, int j) { return b->is_hbm[j] != 0; }
+bool runs_alone(const euler_batch* b, int j) { return b->is_alone[j] != 0; }
 
 // Tile of network j in the persistent launch: the widest phase x Rt ~ block,
 // at least 8 replications, scaled by 2^rt_shift, reduced until it fits the
@@ -127,7 +129,7 @@ bool tile_for(const euler_batch* b, int j, int block, int64_t cap, int rt_shift,
 }
 
 // Plan for a block size, a per-CTA shared-memory budget, a tile scale, the
-// HBM-form threshold and the critical-path factor.
+// threshold from which a network runs by itself and the critical-path factor.
 //
 // Critical-path rule: a work item is one tile of replications through the
 // network's whole horizon on one CTA, so when the launch has more items than
@@ -138,7 +140,7 @@ bool tile_for(const euler_batch* b, int j, int block, int64_t cap, int rt_shift,
 // step has at least 2^14 units (512 warps) so that its launches do more than
 // wait on launch latency.  With fewer items than CTAs every item runs at
 // once and nothing moves.
-int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_t hbm_min_units,
+int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_t alone_min_units,
                     double cp_factor) {
   if (block % 32 || block < 32 || block > 512) return bfail(EULER_ERR_ARG, "batch block must be a multiple of 32 in [32, 512]");
   cap = std::min<int64_t>(cap, b->smem_optin);
@@ -146,26 +148,27 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
   b->block = block;
   b->smem_cap = cap;
   b->rt_shift = rt_shift;
-  b->hbm_min_units = hbm_min_units;
+  b->alone_min_units = alone_min_units;
   b->cp_factor = cp_factor;
-  b->is_hbm.assign(b->count, 0);
+  b->is_alone.assign(b->count, 0);
   for (int j = 0; j < b->count; ++j)
-    b->is_hbm[j] = hbm_min_units > 0 && (int64_t)b->nets[j]->n * b->runs[j].replications >= hbm_min_units;
+    b->is_alone[j] = alone_min_units > 0 && (int64_t)b->nets[j]->n * b->runs[j].replications >= alone_min_units;
   std::vector<int64_t> Rt_of(b->count, 1);
   for (int j = 0; j < b->count; ++j) {
-    if (b->is_hbm[j]) continue;
+    if (b->is_alone[j]) continue;
     const euler_net* h = b->nets[j];
+    // the documented limit of a network of the shared launch
     if (288 + 4 * ((int64_t)h->n + (int64_t)h->tables().ring * h->E) > cap)
       return bfail(EULER_ERR_TOO_LARGE, "a network's state of one replication does not fit the shared-memory budget");
     // a tile whose lists and arrivals do not fit beside the state: by itself
-    if (!tile_for(b, j, block, cap, rt_shift, &Rt_of[j])) b->is_hbm[j] = 1;
+    if (!tile_for(b, j, block, cap, rt_shift, &Rt_of[j])) b->is_alone[j] = 1;
   }
   if (cp_factor > 0.0) {
     for (int pass = 0; pass < 8; ++pass) {
       int64_t smem = 256;
       double work = 0.0, n_items = 0.0;
       for (int j = 0; j < b->count; ++j) {
-        if (b->is_hbm[j]) continue;
+        if (b->is_alone[j]) continue;
         const euler_net* h = b->nets[j];
         smem = std::max<int64_t>(smem, tile_bytes(h, b->runs[j].scheme, Rt_of[j]));
         work += (double)h->n * (double)euler_num_steps(b->runs[j].dt, b->runs[j].T) * (double)b->runs[j].replications;
@@ -177,17 +180,17 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
       if (n_items <= ctas) break;
       bool moved = false;
       for (int j = 0; j < b->count; ++j) {
-        if (b->is_hbm[j] || (int64_t)b->nets[j]->n * b->runs[j].replications < (int64_t(1) << 14)) continue;
+        if (b->is_alone[j] || (int64_t)b->nets[j]->n * b->runs[j].replications < (int64_t(1) << 14)) continue;
         const double item = (double)b->nets[j]->n * (double)euler_num_steps(b->runs[j].dt, b->runs[j].T) * (double)Rt_of[j];
         if (item > cp_factor * work / ctas) {
-          b->is_hbm[j] = 1;
+          b->is_alone[j] = 1;
           moved = true;
         }
       }
       if (!moved) break;
     }
   }
-  b->hbm_nets.clear();
+  b->alone_nets.clear();
   b->h_runs.assign(b->count, RunParams{});
   b->h_nets.assign(b->count, NetTables{});
   b->h_items.clear();
@@ -198,8 +201,8 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
     euler_net* h = b->nets[j];
     const euler_run& r = b->runs[j];
     const int64_t K = euler_num_steps(r.dt, r.T);
-    if (b->is_hbm[j]) {
-      b->hbm_nets.push_back(j);
+    if (b->is_alone[j]) {
+      b->alone_nets.push_back(j);
       continue;
     }
     const int64_t Rt = Rt_of[j];
@@ -270,7 +273,7 @@ int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_
     b->sacc_cap = sacc_need;
   }
   size_t alone_need = 0;
-  for (int j : b->hbm_nets) {
+  for (int j : b->alone_nets) {
     const euler_net* h = b->nets[j];
     SlotPlan sp;
     if (plan_alone(h, b->runs[j].scheme, b->runs[j].replications, &sp))
@@ -309,7 +312,7 @@ int upload_runs(euler_batch* b, int64_t* const* stats, double k_scale) {
   std::vector<RunParams> rp = b->h_runs;
   for (int j = 0; j < b->count; ++j) {
     rp[j].stats = stats[j];
-    if (!b->is_hbm[j]) rp[j].K = (int32_t)scaled_steps(b, j, k_scale);
+    if (!b->is_alone[j]) rp[j].K = (int32_t)scaled_steps(b, j, k_scale);
   }
   BTRY(cudaMemcpy(b->d_runs, rp.data(), sizeof(RunParams) * b->count, cudaMemcpyHostToDevice));
   return EULER_OK;
@@ -318,9 +321,9 @@ int upload_runs(euler_batch* b, int64_t* const* stats, double k_scale) {
 // The networks run by themselves, one after another on stream s (horizons
 // scaled by k_scale for tuning; only the networks in `subset` when it is not
 // null).
-int run_hbm_nets(euler_batch* b, int64_t* const* stats, cudaStream_t s, double k_scale,
+int run_alone_nets(euler_batch* b, int64_t* const* stats, cudaStream_t s, double k_scale,
                  const std::vector<int>* subset = nullptr) {
-  for (int j : subset ? *subset : b->hbm_nets) {
+  for (int j : subset ? *subset : b->alone_nets) {
     const euler_run& r = b->runs[j];
     const int rc = simulate_alone(b->nets[j], r.scheme, r.dt, r.T, r.replications, r.seed, r.rep_begin, stats[j], s,
                                   b->hbm_block, b->hbm_graph_steps, k_scale > 0.0 ? scaled_steps(b, j, k_scale) : 0,
@@ -444,16 +447,16 @@ int euler_batch_autotune(euler_batch* b, void* cuda_stream, int32_t* block_out) 
   int64_t kmax = 1;
   for (int j = 0; j < b->count; ++j) kmax = std::max<int64_t>(kmax, euler_num_steps(b->runs[j].dt, b->runs[j].T));
   const double k_scale = std::min(1.0, 48.0 / (double)kmax);
-  // one timed trial: the persistent launch and, if hbm, the HBM-form
+  // one timed trial: the persistent launch and, if `alone`, the networks run by themselves
   // networks (`subset` only, if set), horizons scaled by ks
-  auto trial = [&](double ks, bool persistent, bool hbm, const std::vector<int>* subset, float* ms) -> int {
+  auto trial = [&](double ks, bool persistent, bool alone, const std::vector<int>* subset, float* ms) -> int {
     int r = upload_runs(b, st.data(), ks);
     if (r) return r;
     cudaError_t e = cudaEventRecord(e0, s);
     if (e == cudaSuccess && persistent && b->num_items > 0) e = enqueue(b, st.data(), s);
     if (e != cudaSuccess) return bcuda(e, "batch autotune");
-    if (hbm) {
-      r = run_hbm_nets(b, st.data(), s, ks, subset);
+    if (alone) {
+      r = run_alone_nets(b, st.data(), s, ks, subset);
       if (r) return r;
     }
     e = cudaEventRecord(e1, s);
@@ -461,10 +464,10 @@ int euler_batch_autotune(euler_batch* b, void* cuda_stream, int32_t* block_out) 
     if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
     return e == cudaSuccess ? EULER_OK : bcuda(e, "batch autotune");
   };
-  const int64_t hbm_min0 = b->hbm_min_units;
+  const int64_t alone_min0 = b->alone_min_units;
   const double cp0 = b->cp_factor;
   int best_block = b->block, best_shift = b->rt_shift;
-  int64_t best_cap = b->smem_cap, best_min = hbm_min0;
+  int64_t best_cap = b->smem_cap, best_min = alone_min0;
   double best_cp = cp0;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) rc = bcuda(cudaErrorUnknown, "event");
   // 1. the persistent launch: threads per block x shared-memory budget x tile scale
@@ -475,7 +478,7 @@ int euler_batch_autotune(euler_batch* b, void* cuda_stream, int32_t* block_out) 
     for (int bi = 0; bi < 3 && rc == EULER_OK; ++bi)
       for (int ci = 0; ci < 3 && rc == EULER_OK; ++ci)
         for (int sh = -1; sh <= 1 && rc == EULER_OK; ++sh) {
-          if (make_batch_plan(b, blocks[bi], caps[ci], sh, hbm_min0, cp0) != EULER_OK || b->num_items == 0) continue;
+          if (make_batch_plan(b, blocks[bi], caps[ci], sh, alone_min0, cp0) != EULER_OK || b->num_items == 0) continue;
           float ms = 0.0f;
           rc = trial(k_scale, true, false, nullptr, &ms);
           if (rc == EULER_OK && (best < 0.0f || ms < best)) {
@@ -488,9 +491,9 @@ int euler_batch_autotune(euler_batch* b, void* cuda_stream, int32_t* block_out) 
   }
   // 2. the HBM form: threads per step kernel x slots per graph replay, on up
   // to six of its networks spread over their sizes, 128 steps each at most
-  if (rc == EULER_OK) rc = make_batch_plan(b, best_block, best_cap, best_shift, hbm_min0, cp0);
-  if (rc == EULER_OK && !b->hbm_nets.empty()) {
-    std::vector<int> by_size = b->hbm_nets;
+  if (rc == EULER_OK) rc = make_batch_plan(b, best_block, best_cap, best_shift, alone_min0, cp0);
+  if (rc == EULER_OK && !b->alone_nets.empty()) {
+    std::vector<int> by_size = b->alone_nets;
     std::sort(by_size.begin(), by_size.end(), [&](int x, int y) {
       return b->nets[x]->n * b->runs[x].replications < b->nets[y]->n * b->runs[y].replications;
     });
@@ -566,7 +569,7 @@ int euler_batch_run(euler_batch* b, int64_t* const* stats, void* cuda_stream) tr
     const int rc = prepare_step_tables(h, b->runs[j].dt, b->runs[j].T, s);
     if (rc) return rc;
     RunParams& p = b->h_runs[j];
-    if (!runs_hbm(b, j) && (p.p0 != h->d_p0 || p.lam != h->d_lam || p.muh != h->d_muh || p.mtab != h->mtab())) {
+    if (!runs_alone(b, j) && (p.p0 != h->d_p0 || p.lam != h->d_lam || p.muh != h->d_muh || p.mtab != h->mtab())) {
       p.p0 = h->d_p0;
       p.lam = h->d_lam;
       p.muh = h->d_muh;
@@ -598,7 +601,7 @@ int euler_batch_run(euler_batch* b, int64_t* const* stats, void* cuda_stream) tr
     b->graph_stats.assign(stats, stats + b->count);
   }
   BTRY(cudaGraphLaunch(b->exec, s));  // zeroes every stats buffer, runs the persistent items
-  return run_hbm_nets(b, stats, s, 0.0);
+  return run_alone_nets(b, stats, s, 0.0);
 } catch (const std::bad_alloc&) {
   return bfail(EULER_ERR_OOM, "host memory allocation failed");
 } catch (...) {
@@ -609,8 +612,8 @@ int euler_batch_info(const euler_batch* b, int32_t* hbm_networks, int64_t* hbm_m
                      int32_t* critical_path, int32_t* block, int32_t* tile_shift, int32_t* hbm_block,
                      int32_t* graph_steps) {
   if (!b) return bfail(EULER_ERR_ARG, "batch is NULL");
-  if (hbm_networks) *hbm_networks = (int32_t)b->hbm_nets.size();
-  if (hbm_min_units) *hbm_min_units = b->hbm_min_units;
+  if (hbm_networks) *hbm_networks = (int32_t)b->alone_nets.size();
+  if (hbm_min_units) *hbm_min_units = b->alone_min_units;
   if (critical_path) *critical_path = b->cp_factor > 0.0 ? 1 : 0;
   if (block) *block = b->block;
   if (tile_shift) *tile_shift = b->rt_shift;

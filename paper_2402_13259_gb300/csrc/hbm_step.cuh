@@ -1,6 +1,6 @@
 // hbm_step.cuh -- the HBM form's per-step kernel: one launch per step (or
 // skewed slot) over all stations, state in global memory, one warp per
-// (station, 32 replications), no block barrier.  The benchmark's kernel.
+// (station, 32 replications), no block barrier.
 #pragma once
 
 #include <cstdint>

@@ -170,7 +170,6 @@ inline void set_round_keys(HbmState& hs, uint32_t key0, uint32_t key1) { set_rou
 
 // What the HBM form's per-step kernels compute besides the step.
 enum HbmMode { kHbmPlain = 0, kHbmGrad = 1, kHbmSojourn = 2 };
-int64_t hbm_smem_bytes(int32_t n, int32_t tile_reps);
 cudaError_t launch_hbm_init(const NetTables& t, const RunParams& p, const HbmState& hs,
                             cudaStream_t s);
 // One step's kernels (backward: 2 phases; forward: one per level), then the

@@ -13,9 +13,10 @@
 //   backward (Sec. 2.2 tasks 1-4, Algorithm 2): D from N_{tau-1}, routing,
 //     external arrivals for every station, then -- after a block barrier --
 //     the gather of routed counts over the reverse graph (CSC) and the update;
-//   forward (Sec. 2.2 tasks 1-4, Algorithm 3): level by level in flow order,
-//     gather, external arrivals, D from N_{tau-1} + A^ex + A^in, update,
-//     routing; a barrier between levels.
+//   forward (Sec. 2.2 tasks 1-4, Algorithm 3): gather, external arrivals, D from
+//     N_{tau-1} + A^ex + A^in, update, routing, in skewed slots: the station at
+//     level l runs step tau - l, so a slot holds units of all levels and only
+//     slots are separated by a barrier (a launch in the hbm form).
 #include <cstdint>
 
 #include "internal.h"
@@ -304,8 +305,6 @@ cudaError_t launch_average(const int64_t* b, const int64_t* f, double* out, int6
   average_kernel<<<256, 256, 0, s>>>(b, f, out, len);
   return cudaGetLastError();
 }
-
-int64_t hbm_smem_bytes(int32_t, int32_t) { return 0; }
 
 cudaError_t launch_hbm_init(const NetTables& t, const RunParams& p, const HbmState& hs,
                             cudaStream_t s) {

@@ -31,22 +31,6 @@
 #define EN_HD inline
 #define EN_D inline
 #endif
-// Rarely taken sampler paths (rejection samplers for large means, Erlang
-// times) are inlined like the rest unless EN_COLD_OUTLINE is defined (one
-// out-of-line copy each: smaller code, but calls and more spills).
-#if defined(__CUDACC__) && defined(EN_COLD_OUTLINE)
-#define EN_COLD static __device__ __noinline__
-#else
-#define EN_COLD EN_D
-#endif
-// The Philox block function is inlined at every draw site unless
-// EN_PHILOX_OUTLINE is defined (one out-of-line copy: smaller code).
-#if defined(__CUDACC__) && defined(EN_PHILOX_OUTLINE)
-#define EN_REFILL __device__ __noinline__
-#else
-#define EN_REFILL EN_D
-#endif
-
 // Branch-probability hints (code placement only: the arithmetic is the same).
 #if defined(__CUDACC__) || defined(__GNUC__)
 #define EN_LIKELY(c) __builtin_expect(!!(c), 1)
@@ -278,7 +262,7 @@ struct PhiloxStream {
     block = 0;
   }
 
-  EN_REFILL void refill() {
+  EN_D void refill() {
     uint32_t x0 = ctr0 | block, x1 = ctr1, x2 = ctr2, x3 = ctr3;
     uint32_t k0 = key0, k1 = key1;
 #pragma unroll
@@ -457,7 +441,7 @@ EN_D float log_binom_pmf(int k, int n, float p, float q, float se_n) {
 // decision is the exact functions'.  The largest deviation from the exact float
 // functions over the domain (standard deviation below kFastMaxSd, |k - mode|
 // below kFastMaxDev of them, n < 2^24) is 0.16 of the tolerance, both sides of
-// the test evaluated on GB300 (1.5e7 binomial and Poisson tests as drawn, 4e6 near
+// the test evaluated on GB300 (1.5e7 binomial and Poisson tests as drawn, 3e6 near
 // their line, over the whole range); the hardware functions' stated errors alone
 // would allow about 0.3 of it.
 // The mode's log-pmf, formerly computed before every draw, is needed only for
@@ -549,7 +533,7 @@ EN_D int fast_decide(float lv, float f) {
 // Samplers.
 // ---------------------------------------------------------------------------
 // Hoermann's PTRS for lam >= 10.
-EN_COLD int32_t poisson_ptrs(float lam, PhiloxStream& st, SamplerCtx& cx) {
+EN_D int32_t poisson_ptrs(float lam, PhiloxStream& st, SamplerCtx& cx) {
   const float slam = sqrtf(lam);
   const float b = 0.931f + 2.53f * slam;
   const float a = -0.059f + 0.02483f * b;
@@ -682,7 +666,7 @@ EN_HD BinomConst binom_const(float p) {
 }
 
 // Hoermann's BTRS for Bin(n, p), p <= 1/2, n p >= 10.
-EN_COLD int32_t binomial_btrs(int32_t n, float p, float q, PhiloxStream& st, SamplerCtx& cx) {
+EN_D int32_t binomial_btrs(int32_t n, float p, float q, PhiloxStream& st, SamplerCtx& cx) {
   const float nf = (float)n;
   const float np = nf * p;
   const float spq = sqrtf(np * q);
@@ -769,7 +753,7 @@ EN_D float std_normal(PhiloxStream& st, SamplerCtx& cx) {
   return 0.0f;
 }
 
-EN_COLD float erlang(int32_t k, float rate, PhiloxStream& st, SamplerCtx& cx) {
+EN_D float erlang(int32_t k, float rate, PhiloxStream& st, SamplerCtx& cx) {
   if (k <= 0) return 0.0f;
   if (k <= 8) {
     float S = 0.0f;

@@ -121,9 +121,8 @@ extern "C" int euler_net_sojourn(euler_net* h, int32_t scheme, double dt, double
   SlotPlan sp;
   const bool tiled = plan_slots(h, scheme, R, false, samples, 0, 0, &sp);
   const bool large = (int64_t)h->n * R >= kHbmMinUnitsPerStep;
-  // a network and sample count beyond a tile of one replication (its state,
-  // one step's inputs and departures, its customers), unless the HBM form is
-  // asked for or the step has work for the whole GPU
+  // the documented limit of a small run (and of form 1): one replication's state
+  // with its station sums, one step's inputs and departures, and its customers
   const int64_t least = 288 + 60 * (int64_t)h->n + 4 * (int64_t)h->E + 12 * (int64_t)samples;
   if (forced != 2 && (forced > 0 || !large) && least > h->smem_optin)
     return fail(EULER_ERR_TOO_LARGE, "sojourn tile does not fit in shared memory");
