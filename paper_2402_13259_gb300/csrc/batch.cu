@@ -490,10 +490,15 @@ int euler_batch_autotune(euler_batch* b, void* cuda_stream, int32_t* block_out) 
         }
   }
   // 2. the HBM form: threads per step kernel x slots per graph replay, on up
-  // to six of its networks spread over their sizes, 128 steps each at most
+  // to six of the networks that take it spread over their sizes, 128 steps each
+  // at most
   if (rc == EULER_OK) rc = make_batch_plan(b, best_block, best_cap, best_shift, alone_min0, cp0);
-  if (rc == EULER_OK && !b->alone_nets.empty()) {
-    std::vector<int> by_size = b->alone_nets;
+  std::vector<int> by_size;
+  SlotPlan unused;
+  if (rc == EULER_OK)
+    for (int j : b->alone_nets)
+      if (!plan_alone(b->nets[j], b->runs[j].scheme, b->runs[j].replications, &unused)) by_size.push_back(j);
+  if (!by_size.empty()) {
     std::sort(by_size.begin(), by_size.end(), [&](int x, int y) {
       return b->nets[x]->n * b->runs[x].replications < b->nets[y]->n * b->runs[y].replications;
     });
@@ -522,7 +527,7 @@ int euler_batch_autotune(euler_batch* b, void* cuda_stream, int32_t* block_out) 
     b->hbm_block = bb;
     b->hbm_graph_steps = bg;
   }
-  // 3. which networks take the HBM form: the n R threshold x the
+  // 3. which networks run by themselves: the n R threshold x the
   // critical-path rule (on / off), the whole batch
   if (rc == EULER_OK) {
     const int64_t mins[4] = {int64_t(1) << 16, int64_t(1) << 18, int64_t(1) << 20, 0};

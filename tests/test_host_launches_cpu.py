@@ -306,3 +306,25 @@ for R, K in ((30000, 10000), (30000, 1000), (300000, 1000), (10000, 400000)):
     assert (len(got) > 1) == (R * K * 100 > 2e10 and tiles > p["grid"]), (R, K, got)
     h.close()
 """)
+
+
+def test_autotuner_times_step_kernels_where_they_run(host):
+    """The per-step kernels' launch shape is chosen on networks that take them,
+    and left alone where none does."""
+    host("""
+def tuned(x, R, scheme):
+    hs = [net(x), net(chain(3))]
+    runs = (Bd._Run * 2)(Bd._Run(scheme, 0.1, 20.0, R, 5, 0), Bd._Run(0, 0.1, 2.0, 80, 5, 0))
+    b = C.c_void_p()
+    assert L.euler_batch_create(C.byref(b), (C.c_void_p * 2)(*[x._h for x in hs]), runs, 2) == 0
+    log()
+    assert L.euler_batch_autotune(b, None, None) == 0
+    blocks = set(y.split("block=")[1] for y in log().splitlines() if y.startswith("hbm_phase_kernel"))
+    v = [C.c_int32() for _ in range(7)]; v[1] = C.c_int64()
+    L.euler_batch_info(b, *[C.byref(y) for y in v])
+    L.euler_batch_destroy(b)
+    return blocks, v[5].value, v[6].value
+for _ in range(4):  # the stand-in's times favour another shape each time
+    assert tuned(chain(100), 10000, 0) == (set(), 256, 32)
+assert tuned(two_wide(100), 5000, 1)[0] == {"128", "256"}
+""")
