@@ -36,10 +36,14 @@ sys.path.insert(0, ROOT)
 METRIC = "station-step updates/s per GB300 (fwd/bwd Euler), % of binding roofline"
 UNIT = "station-step updates/s"
 LANES_PER_SM = 128  # instruction issue: 4 schedulers x 32 lanes per clock
-# DRAM bytes of one simulate call (mean of the two schemes) from an ncu
-# capture, valid only for the kernel sources with this hash and the launch
-# forms listed; none is held for the present sources, so null is reported.
-TRAFFIC = {"hash": None, "forms": [1, 1], "bytes_per_call": None}
+# DRAM bytes of one simulate call (mean of the two schemes) from an ncu capture,
+# valid only for the kernel sources with this hash and the launch forms listed;
+# reported as null otherwise.  None is held for the per-step kernels; the
+# persistent kernel's one launch at full size: 0.933 + 0.030 MB read and written
+# backward, 1.108 + 0.027 MB forward.
+TRAFFIC = {"hash": None, "forms": [2, 2], "bytes_per_call": None}
+TRAFFIC_PERSISTENT = {"hash": "b0aa5b020c9c53f6", "forms": [1, 1],
+                      "bytes_per_call": 0.5 * (933120 + 30208 + 1107968 + 27136)}
 
 
 def sm_count(device: int = 0) -> int:
@@ -767,12 +771,13 @@ def main():
         sm_max = clk.get("sm_max_mhz") or getattr(torch.cuda.get_device_properties(local), "clock_rate", 0) / 1e3
         sms = sm_count(local)
         peak = sms * LANES_PER_SM * sm_max * 1e6
-        valid = TRAFFIC["hash"] == kernel_hash() and TRAFFIC.get("forms") == [plans["backward"]["form"],
-                                                                             plans["forward"]["form"]]
+        ran = {"hash": kernel_hash(), "forms": [plans["backward"]["form"], plans["forward"]["form"]]}
+        traffic = next((t["bytes_per_call"] for t in (TRAFFIC, TRAFFIC_PERSISTENT)
+                        if all(t[k] == ran[k] for k in ran)), None)
         hbm = plans["backward"]["form"] == 2
         roof = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tops/s",
                 "frac": achieved / peak,
-                "traffic": TRAFFIC["bytes_per_call"] if valid else None,
+                "traffic": traffic,
                 "kernel": "hbm_phase_kernel (per-step kernels of one simulate call, CUDA graph)" if hbm
                           else "persistent_kernel",
                 "launch": "one euler_net_simulate call per scheme (kernel time" +
