@@ -143,7 +143,7 @@ bool tile_for(const euler_batch* b, int j, int block, int64_t cap, int rt_shift,
 int make_batch_plan(euler_batch* b, int block, int64_t cap, int rt_shift, int64_t alone_min_units,
                     double cp_factor) {
   if (block % 32 || block < 32 || block > 512) return bfail(EULER_ERR_ARG, "batch block must be a multiple of 32 in [32, 512]");
-  cap = std::min<int64_t>(cap, b->smem_optin);
+  cap = std::min<int64_t>(cap, b->smem_optin - kBatchStaticSmem);
   b->planned = false;
   b->block = block;
   b->smem_cap = cap;

@@ -98,6 +98,16 @@ inline bool draws_in_place(int64_t tasks, int64_t warps) { return 2 * tasks <= 3
 constexpr int kSlotThreads = 1024;  // most threads per block (the register budget: 64)
 constexpr int kSlotResGradThreads = 512;  // of the resident gradient variant
 
+// Dynamic shared memory that a launch of `fn` may ask for: always all that a
+// block can have beside the kernel's static memory.  The limit belongs to the
+// function, so one set to a call's own need could be lowered by another thread's
+// call between this call's setting and its launch.
+constexpr int kSmemPerBlock = 227 * 1024;
+constexpr int kBatchStaticSmem = 512;  // the work item's tables (batch_kernel)
+inline cudaError_t allow_smem(const void* fn, int static_smem = 0) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemPerBlock - static_smem);
+}
+
 // Batched form: one persistent launch over (network, tile) work items.
 cudaError_t batch_occupancy(int block, int smem, int* blocks_per_sm);
 cudaError_t launch_batch(int scheme, bool ext, const NetTables* nets, const RunParams* runs, const int2* items,

@@ -115,6 +115,7 @@ template <int SCHEME, bool EXT>
 __global__ void __launch_bounds__(kSlotThreads, 1)
     batch_kernel(const NetTables* nets, const RunParams* runs, const int2* items, int num_items,
                  int* next_item, unsigned long long* acc_scratch, int64_t acc_slot_len) {
+  static_assert(sizeof(NetTables) + sizeof(RunParams) + 64 <= kBatchStaticSmem, "static shared memory");
   __shared__ int s_item;
   __shared__ __align__(16) unsigned char t_raw[sizeof(NetTables)], p_raw[sizeof(RunParams)];
   const NetTables& t = *reinterpret_cast<const NetTables*>(t_raw);
@@ -229,10 +230,11 @@ const void* batch_fn(int scheme, bool ext) {
 }
 
 // Occupancy of the tightest of a set of instantiations at (block, smem).
-cudaError_t min_occupancy(const void* const* fns, int count, int block, int smem, int* blocks_per_sm) {
+cudaError_t min_occupancy(const void* const* fns, int count, int block, int smem, int* blocks_per_sm,
+                          int static_smem = 0) {
   int best = 1 << 30;
   for (int k = 0; k < count; ++k) {
-    cudaError_t e = cudaFuncSetAttribute(fns[k], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(fns[k], static_smem);
     int v = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, fns[k], block, smem);
     if (e != cudaSuccess) return e;
@@ -242,8 +244,9 @@ cudaError_t min_occupancy(const void* const* fns, int count, int block, int smem
   return cudaSuccess;
 }
 
-cudaError_t launch_fn(const void* fn, void** args, int grid, int block, int smem, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+cudaError_t launch_fn(const void* fn, void** args, int grid, int block, int smem, cudaStream_t s,
+                      int static_smem = 0) {
+  cudaError_t e = allow_smem(fn, static_smem);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, (size_t)smem, s);
 }
@@ -264,14 +267,14 @@ cudaError_t launch_persistent(const NetTables& t, const RunParams& p, int mode, 
 
 cudaError_t batch_occupancy(int block, int smem, int* blocks_per_sm) {
   const void* fns[4] = {batch_fn(0, false), batch_fn(1, false), batch_fn(0, true), batch_fn(1, true)};
-  return min_occupancy(fns, 4, block, smem, blocks_per_sm);
+  return min_occupancy(fns, 4, block, smem, blocks_per_sm, kBatchStaticSmem);
 }
 
 cudaError_t launch_batch(int scheme, bool ext, const NetTables* nets, const RunParams* runs,
                          const int2* items, int num_items, int* next_item, unsigned long long* acc_scratch,
                          int64_t acc_slot_len, int grid, int block, int smem, cudaStream_t s) {
   void* args[] = {&nets, &runs, &items, &num_items, &next_item, &acc_scratch, &acc_slot_len};
-  return launch_fn(batch_fn(scheme, ext), args, grid, block, smem, s);
+  return launch_fn(batch_fn(scheme, ext), args, grid, block, smem, s, kBatchStaticSmem);
 }
 
 cudaError_t launch_grad_reduce(int32_t n, int64_t R, double dt, const int64_t* stats,

@@ -220,7 +220,7 @@ int64_t pipeline_smem_bytes(int32_t n, int32_t E) {
 
 cudaError_t pipeline_occupancy(int scheme, int block, int smem, int* blocks_per_sm) {
   const void* fn = scheme == 0 ? (const void*)pipeline_kernel<0> : (const void*)pipeline_kernel<1>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, block, smem);
 }
@@ -228,7 +228,7 @@ cudaError_t pipeline_occupancy(int scheme, int block, int smem, int* blocks_per_
 cudaError_t launch_pipeline(const NetTables& t, const RunParams& p, const PipePlan& pp, int grid,
                             int smem, cudaStream_t s) {
   const void* fn = p.scheme == 0 ? (const void*)pipeline_kernel<0> : (const void*)pipeline_kernel<1>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   const int block = 32 * pp.W;
   if (p.scheme == 0)

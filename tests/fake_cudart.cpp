@@ -6,12 +6,14 @@
 // violation or a launch is a line of the log.
 #include <dlfcn.h>
 #include <sys/mman.h>
+#include <unistd.h>
 
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 
 #include <cuda_runtime.h>
@@ -34,6 +36,12 @@ std::string& text() {
   static auto* s = new std::string();
   return *s;
 }
+std::map<const void*, int>& smem_limit() {
+  static auto* m = new std::map<const void*, int>();
+  return *m;
+}
+std::recursive_mutex all;  // several threads may call
+#define LOCKED std::lock_guard<std::recursive_mutex> lock_(all)
 long long fail_from = 0, allocs = 0;  // allocations numbered from fail_from on fail (0: none)
 
 void line(const char* fmt, const char* what, long long a, long long b) {
@@ -77,6 +85,8 @@ void check_hbm(const NetTables* t, const RunParams& p, const HbmState& hs, const
 }
 
 cudaError_t launched(const void* fn, dim3 grid, dim3 block, void** a, size_t smem) {
+  LOCKED;
+  if (smem > 48 * 1024 && (int)smem > smem_limit()[fn]) return cudaErrorInvalidValue;
   const std::string name = kernels()[fn];
   auto is = [&](const char* s) { return name.find(s) != std::string::npos; };
   auto net = [&](int k) { return static_cast<const NetTables*>(a[k]); };
@@ -145,6 +155,7 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, voi
 }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
+  LOCKED;
   *p = nullptr;
   if (fail_from > 0 && ++allocs >= fail_from) return cudaErrorMemoryAllocation;
   void* q = mmap(nullptr, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
@@ -154,6 +165,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
   return cudaSuccess;
 }
 cudaError_t cudaFree(void* p) {
+  LOCKED;
   if (!p) return cudaSuccess;
   auto it = blocks().find((uintptr_t)p);
   if (it == blocks().end()) {
@@ -165,12 +177,14 @@ cudaError_t cudaFree(void* p) {
   return cudaSuccess;
 }
 cudaError_t cudaMemset(void* p, int v, size_t n) {
+  LOCKED;
   within(p, (int64_t)n, "memset");
   if (n <= 4096 && blocks().count((uintptr_t)p)) std::memset(p, v, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { return cudaMemset(p, v, n); }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind k) {
+  LOCKED;
   within(k == cudaMemcpyDeviceToHost ? s : d, (int64_t)n, "memcpy");
   if (k == cudaMemcpyDeviceToHost) std::memset(d, 0, n);
   return cudaSuccess;
@@ -192,7 +206,15 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* v, const void*, i
   *v = by_regs < by_smem ? by_regs : by_smem;
   return cudaSuccess;
 }
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute, int bytes) {
+  usleep(20);  // another thread's call may come between this one and the launch
+  LOCKED;
+  // what a function's static memory leaves (batch_kernel: its work item's tables)
+  const int most = 227 * 1024 - (kernels()[fn].find("batch_kernel") != std::string::npos ? 448 : 0);
+  if (bytes > most) return cudaErrorInvalidValue;
+  smem_limit()[fn] = bytes;
+  return cudaSuccess;
+}
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {

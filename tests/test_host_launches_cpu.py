@@ -328,3 +328,43 @@ for _ in range(4):  # the stand-in's times favour another shape each time
     assert tuned(chain(100), 10000, 0) == (set(), 256, 32)
 assert tuned(two_wide(100), 5000, 1)[0] == {"128", "256"}
 """)
+
+
+def test_threads_on_different_networks(host):
+    """Calls of several threads, each on its own handle, do not lower one
+    another's shared-memory limits."""
+    host("""
+import threading
+def work(n, R, scheme, out):
+    h = net(chain(n))
+    s = dev(8 * Bd.stats_len(n, R))
+    for _ in range(150):
+        rc = L.euler_net_simulate(h._h, scheme, 0.1, 1.0, R, 1, 0, s, None)
+        if rc:
+            out.append((n, rc, L.euler_net_last_error().decode()))
+            break
+    h.close()
+for form_scheme in (0, 1):
+    bad = []
+    ts = [threading.Thread(target=work, args=(n, R, form_scheme, bad)) for n, R in ((100, 10000), (100, 4000), (90, 9000))]
+    [t.start() for t in ts]; [t.join() for t in ts]
+    assert not bad, bad
+""")
+
+
+def test_batch_tile_leaves_room_for_its_tables(host):
+    """The largest shared-memory budget of the autotuner leaves room for the
+    work item's tables, which are static memory of the batched kernel."""
+    host("""
+for n in (1887, 1890, 943, 944):  # 8 and 16 replications: 232,048 to 232,448 bytes
+    hs = [net(chain(n))]
+    runs = (Bd._Run * 1)(Bd._Run(0, 0.1, 1.0, 150, 5, 0))
+    b = C.c_void_p()
+    assert L.euler_batch_create(C.byref(b), (C.c_void_p * 1)(hs[0]._h), runs, 1) == 0
+    st = (C.c_void_p * 1)(dev(8 * Bd.stats_len(n, 150)))
+    for _ in range(6):  # the stand-in's times favour another shape each time
+        assert L.euler_batch_autotune(b, None, None) == 0, L.euler_net_last_error()
+        assert L.euler_batch_run(b, st, None) == 0, L.euler_net_last_error()
+    L.euler_batch_destroy(b)
+    hs[0].close()
+""")
