@@ -45,6 +45,7 @@ void eulernet::set_last_error(const char* msg) { g_last_error = msg; }
 namespace {
 
 int cuda_fail(cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here: no later launch check, ours or the caller's, may take it for its own
   g_last_error = std::string("CUDA error in ") + where + ": " + cudaGetErrorString(e);
   return e == cudaErrorMemoryAllocation ? EULER_ERR_OOM : EULER_ERR_CUDA;
 }

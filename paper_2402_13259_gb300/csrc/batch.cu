@@ -87,6 +87,7 @@ int bfail(int code, const std::string& msg) {
 }
 
 int bcuda(cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here, not by a later launch check
   std::string m = std::string("CUDA error in ") + where + ": " + cudaGetErrorString(e);
   set_last_error(m.c_str());
   return e == cudaErrorMemoryAllocation ? EULER_ERR_OOM : EULER_ERR_CUDA;

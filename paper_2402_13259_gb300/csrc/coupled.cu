@@ -35,6 +35,7 @@ int fail(int code, const char* msg) {
 }
 
 int cuda_fail(cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here, not by a later launch check
   set_last_error((std::string("CUDA error in ") + where + ": " + cudaGetErrorString(e)).c_str());
   return e == cudaErrorMemoryAllocation ? EULER_ERR_OOM : EULER_ERR_CUDA;
 }

@@ -66,6 +66,11 @@ int noalloc_fail(int code, const char* msg) {
   return code;
 }
 
+int noalloc_cuda(cudaError_t e) {
+  cudaGetLastError();  // reported here, not by a later launch check
+  return noalloc_fail(EULER_ERR_CUDA, cudaGetErrorString(e));
+}
+
 // Host staging for the per-step tables: a fixed buffer, refilled chunk by
 // chunk (a copy from pageable memory returns once the data is staged).
 constexpr int kStage = 4096;
@@ -124,14 +129,14 @@ extern "C" EULERNET_API int euler_net_simulate_noalloc(euler_net* h, int32_t sch
 
   int device = 0;
   cudaError_t e = cudaGetDevice(&device);
-  if (e != cudaSuccess) return noalloc_fail(EULER_ERR_CUDA, cudaGetErrorString(e));
+  if (e != cudaSuccess) return noalloc_cuda(e);
   if (device != h->device)
     return noalloc_fail(EULER_ERR_ARG, "the handle belongs to another device than the current one");
   unsigned char* base = nullptr;
   e = scratch_address(device, &base);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(stats, 0, sizeof(int64_t) * (size_t)euler_stats_len(h->n, R), s);
-  if (e != cudaSuccess) return noalloc_fail(EULER_ERR_CUDA, cudaGetErrorString(e));
+  if (e != cudaSuccess) return noalloc_cuda(e);
   if (R == 0) return EULER_OK;
 
   // per-call tables, computed by the same host functions as euler_net_simulate's
@@ -189,7 +194,7 @@ extern "C" EULERNET_API int euler_net_simulate_noalloc(euler_net* h, int32_t sch
   }
   unsigned* d_err = reinterpret_cast<unsigned*>(base);
   if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(unsigned), s);
-  if (e != cudaSuccess) return noalloc_fail(EULER_ERR_CUDA, cudaGetErrorString(e));
+  if (e != cudaSuccess) return noalloc_cuda(e);
 
   RunParams p;
   p.p0 = d_p0;
@@ -228,6 +233,6 @@ extern "C" EULERNET_API int euler_net_simulate_noalloc(euler_net* h, int32_t sch
     fold_error_kernel<<<1, 1, 0, s>>>(d_err, h->d_err);  // report through euler_net_status
     e = cudaGetLastError();
   }
-  if (e != cudaSuccess) return noalloc_fail(EULER_ERR_CUDA, cudaGetErrorString(e));
+  if (e != cudaSuccess) return noalloc_cuda(e);
   return EULER_OK;
 }

@@ -44,6 +44,7 @@ int fail(int code, const char* msg) {
 }
 
 int cuda_fail(cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here, not by a later launch check
   char buf[256];
   std::snprintf(buf, sizeof buf, "%s: %s", where, cudaGetErrorString(e));
   set_last_error(buf);

@@ -42,6 +42,8 @@ std::map<const void*, int>& smem_limit() {
 }
 std::recursive_mutex all;  // several threads may call
 #define LOCKED std::lock_guard<std::recursive_mutex> lock_(all)
+thread_local cudaError_t last_error = cudaSuccess;  // kept until it is asked for
+cudaError_t failed(cudaError_t e) { return last_error = e; }
 long long fail_from = 0, allocs = 0;  // allocations numbered from fail_from on fail (0: none)
 
 void line(const char* fmt, const char* what, long long a, long long b) {
@@ -86,7 +88,7 @@ void check_hbm(const NetTables* t, const RunParams& p, const HbmState& hs, const
 
 cudaError_t launched(const void* fn, dim3 grid, dim3 block, void** a, size_t smem) {
   LOCKED;
-  if (smem > 48 * 1024 && (int)smem > smem_limit()[fn]) return cudaErrorInvalidValue;
+  if (smem > 48 * 1024 && (int)smem > smem_limit()[fn]) return failed(cudaErrorInvalidValue);
   const std::string name = kernels()[fn];
   auto is = [&](const char* s) { return name.find(s) != std::string::npos; };
   auto net = [&](int k) { return static_cast<const NetTables*>(a[k]); };
@@ -157,9 +159,9 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, voi
 cudaError_t cudaMalloc(void** p, size_t n) {
   LOCKED;
   *p = nullptr;
-  if (fail_from > 0 && ++allocs >= fail_from) return cudaErrorMemoryAllocation;
+  if (fail_from > 0 && ++allocs >= fail_from) return failed(cudaErrorMemoryAllocation);
   void* q = mmap(nullptr, n ? n : 1, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
-  if (q == MAP_FAILED) return cudaErrorMemoryAllocation;
+  if (q == MAP_FAILED) return failed(cudaErrorMemoryAllocation);
   blocks()[(uintptr_t)q] = n;
   *p = q;
   return cudaSuccess;
@@ -170,7 +172,7 @@ cudaError_t cudaFree(void* p) {
   auto it = blocks().find((uintptr_t)p);
   if (it == blocks().end()) {
     line("VIOLATION %s: %lld %lld\n", "free of an address not allocated", 0, 0);
-    return cudaErrorInvalidValue;
+    return failed(cudaErrorInvalidValue);
   }
   munmap(p, it->second ? it->second : 1);
   blocks().erase(it);
@@ -211,11 +213,15 @@ cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute, int bytes) {
   LOCKED;
   // what a function's static memory leaves (batch_kernel: its work item's tables)
   const int most = 227 * 1024 - (kernels()[fn].find("batch_kernel") != std::string::npos ? 448 : 0);
-  if (bytes > most) return cudaErrorInvalidValue;
+  if (bytes > most) return failed(cudaErrorInvalidValue);
   smem_limit()[fn] = bytes;
   return cudaSuccess;
 }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = last_error;
+  last_error = cudaSuccess;
+  return e;
+}
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
   *s = (cudaStream_t)0x10;
