@@ -29,7 +29,7 @@ struct Worst { float binom, pois; unsigned long long nb, np, decided, wrong; };
 
 __device__ void put(float* a, float v) { atomicMax(reinterpret_cast<int*>(a), __float_as_int(v)); }  // v >= 0
 
-__device__ void judge(float lv_fast, float f, float lv, float ex, float* worst, Worst* w) {
+__device__ void weigh(float lv_fast, float f, float lv, float ex, float* worst, Worst* w) {
   const float tol = fmaf(kFastRel, fabsf(f), kFastTol);
   put(worst, (float)(fabs(((double)lv_fast - (double)f) - ((double)lv - (double)ex)) / (double)tol));
   const int dec = fast_decide(lv_fast, f);
@@ -73,7 +73,7 @@ __global__ void probe(int mode, uint32_t seed, Worst* w) {
           if (v >= 0x1p-24f && v < 1.0f) {  // a uniform
             const float se = stirling_err(nf);
             const float ex = log_binom_pmf(k, n, p, q, se) - log_binom_pmf(md, n, p, q, se);
-            judge(fast_log((v * alpha) * fast_rcp(fmaf(a, fast_rcp(us * us), b))), f,
+            weigh(fast_log((v * alpha) * fast_rcp(fmaf(a, fast_rcp(us * us), b))), f,
                   fm::log_pos(v * alpha / g), ex, &w->binom, w);
             atomicAdd(&w->nb, 1ull);
           }
@@ -92,7 +92,7 @@ __global__ void probe(int mode, uint32_t seed, Worst* w) {
         float V = a2;
         if (mode == 1) V = expf(f + 0.02f * (a2 - 0.5f)) * g / ia;
         if (V >= 0x1p-24f && V < 1.0f) {
-          judge(fast_log((V * ia) * fast_rcp(fmaf(a, fast_rcp(us * us), b))), f, fm::log_pos(V * ia / g),
+          weigh(fast_log((V * ia) * fast_rcp(fmaf(a, fast_rcp(us * us), b))), f, fm::log_pos(V * ia / g),
                 log_pois_pmf(k, lam), &w->pois, w);
           atomicAdd(&w->np, 1ull);
         }
